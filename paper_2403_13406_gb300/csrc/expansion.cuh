@@ -1,0 +1,387 @@
+// expansion.cuh -- the entropic relaxation parameter from the expansion of the entropy about the
+// equilibrium.
+//
+// With B(t) = sum_k B_k(t delta_k) (systems.cuh) the root t* > 0 of B(t) = B(-1) is all that the
+// relaxation needs.  B(t) = c_2 t^2 + c_3 t^3 + ..., and the coefficients have closed forms, so a
+// smooth cell needs no evaluation of B: dividing B(t) - B(-1) by t + 1 leaves
+//   H(e) = sum_n c_n P_n(1 + e) = 0,  P_n(t) = (t^n - (-1)^n) / (t + 1) = t P_{n-1}(t) - (-1)^n,  P_1 = 1,
+// whose root e = t* - 1 = -c_3 / c_2 + ... has full relative precision however close the cell is to
+// equilibrium: B(1) - B(-1), in which all digits cancel there, is never formed.
+//
+// Coefficients, with q = delta / f in the smooth limit:
+//  - scalar systems: d B_k / d h = 2 h / (D (1 + sqrt(1 + x))) with D = D2_k, x = b12_k h / D^2, and
+//    2 / (1 + sqrt(1 + x)) = sum_n C_n (-x / 4)^n with the Catalan numbers C_n, hence
+//    c_{n+2} = C_n / (n + 2) sum_k (delta_k^2 / D_k) y_k^n,  y_k = -b12_k delta_k / (4 D_k^2).
+//  - shallow water: a population is a function of eta = h_1 / f_1, R = sign (h_d - v_d h_1) / (f_1 c) and
+//    kappa = g h / (2 c^2) alone (c = nu + sign v_d; f_1 its equilibrium depth).  With beta = sign b / c
+//    (b the dual velocity's deviation), along the axis B_k / (f_1 c^2) is the stationary value over beta of
+//      Psi(beta) = kappa (eta + beta)^2 / (1 - beta) - R beta - (1 + eta) beta^2 / 2,
+//    and across it the kinetic energy adds (h_t - v_t h_1)^2 / (2 f_1 (1 + eta)).  Psi is stationary, so beta to
+//    order t^2 (beta_1, beta_2) gives B_k through t^5.
+//
+// The terms left out are bounded by the `size` of the cell, the ratio of successive terms: up to
+// Expansion::most the root of the truncated H is the root to the rounding of omega.  Rougher cells
+// take rough_root: Newton on B(t) - B(-1) from the truncated root, with B in the forms above (for
+// shallow water z = (eta + beta) / (1 - beta), (1 + z)(1 - beta) = 1 + eta, turns the stationarity of Psi into a
+// cubic in z), and what that does not certify, the general safeguarded search (entropic_omega).
+// Worst error of omega over 300 000 random cells per system (deviations of 1e-6 ... 0.5 of f), against a
+// bisection in long double: the expansion up to `most` 3e-7 in FP32 and 4e-16 in FP64, Newton on the closed
+// form 1e-6 (1.7e-5 next to the domain's edge) and 2e-15 (5e-14).
+//
+// The root-find bounds every entropic kernel (instruction issue in FP32, the FP64 pipe, 2 lanes a clock
+// and SM, in FP64).  Two evaluations of B by inner Newton solves, a quartic model through them and its
+// certificate took 652 thread instructions per 1D shallow-water cell-stage in all; with the expansion 305.
+// Before -> after: 1D shallow water N = 2^20, FP32, 409 -> 186 us per step; 2D Burgers 4096^2, FP32, 296 -> 141 us
+// per stage; 1D shallow water N = 100003, FP64, 3.26 -> 0.82 ms per step.
+#pragma once
+
+#include "systems.cuh"
+
+namespace eslbm {
+
+// Reciprocal and square root of normal positive numbers to about one unit in the last place: the
+// hardware's approximation, in FP64 with one third-order step of Newton's iteration for 1/x (relative
+// error e -> e^3) and of the binomial series for 1/sqrt(x) (e -> 5/16 e^3).
+__host__ __device__ __forceinline__ float rcp_fast(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+__host__ __device__ __forceinline__ double rcp_fast(double x)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+#else
+    return 1.0 / x;
+#endif
+}
+__host__ __device__ __forceinline__ float sqrt_fast(float x)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return sqrtf(x);
+#endif
+}
+__host__ __device__ __forceinline__ double sqrt_fast(double x)
+{
+#ifdef __CUDA_ARCH__
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double s = x * r;
+    const double e = fma(-s, r, 1.0);
+    return fma(s, e * fma(e, 0.375, 0.5), s);
+#else
+    return sqrt(x);
+#endif
+}
+template <class R> struct Eps;
+template <> struct Eps<float> { static constexpr float value = 1.1920929e-7f; };
+template <> struct Eps<double> { static constexpr double value = 2.220446049250313e-16; };
+
+// Root e of H(e) with c[n] the coefficient of t^(n + 2), N of them: the quadratic model of H about 0 (exact to
+// e^5 relative to c_2), then in FP64 `steps` Newton steps on all of H.
+template <class R, int N> __host__ __device__ __forceinline__ R expansion_root(const R *c, int steps)
+{
+    const R rc = rcp_fast(c[0]);
+    R r[N];
+#pragma unroll
+    for (int n = 1; n < N; ++n) r[n] = c[n] * rc;
+    // H and its first two derivatives at e = 0: P_n(1), P_n'(1), P_n''(1) / 2 up to n = 7
+    R h0 = r[1], h1 = R(1) + r[1] + R(2) * r[2], h2 = r[1] + R(2) * r[2];
+    if constexpr (N > 3) {
+        h0 += r[3];
+        h1 += R(2) * r[3];
+        h2 += R(4) * r[3];
+    }
+    if constexpr (N > 4) h1 += R(3) * r[4];
+    if constexpr (N > 5) h0 += r[5];
+    const R g = rcp_fast(h1);
+    R e = -h0 * g;
+    e = -(h0 + h2 * e * e) * g;
+    for (int i = 0; i < steps; ++i) {
+        const R t = R(1) + e;
+        R p = R(1) + e * t, H = e + r[1] * p;
+        R sgn = R(-1);
+#pragma unroll
+        for (int n = 2; n < N; ++n) {
+            p = t * p + sgn;
+            H += r[n] * p;
+            sgn = -sgn;
+        }
+        e -= H * rcp_fast(h1 + R(2) * h2 * e);
+    }
+    return e;
+}
+
+// Expansion<Sys, R>: build(P, u, delta) computes the coefficients c[0 .. N) of t^2 ... and `size`, the
+// scale of successive terms; false outside the domain or for non-finite data.
+template <class Sys, class R> struct Expansion;
+
+template <int DIM, class R> struct Expansion<Scalar<DIM, true>, R> {
+    static constexpr int Q = Lattice<DIM>::Q;
+    static constexpr int N = sizeof(R) == 4 ? 6 : 8;
+    static constexpr int STEPS = sizeof(R) == 4 ? 0 : 1;
+    // largest size at which the terms left out (95 y^7 of c_2 in FP32, 286 y^8 in FP64) and the model root's
+    // own error (y^5 / 4; in FP64 after one Newton step y^7) are below the rounding of omega; beyond most_rough
+    // (4 y -> 1: the edge of the domain) the closed form does not help
+    static constexpr R most = sizeof(R) == 4 ? R(0.04) : R(0.004);
+    static constexpr R most_rough = R(0.2);
+    R c[N], size;
+    R a[Q], y[Q];
+
+    __host__ __device__ __forceinline__ bool build(const ParamsR<R> &P, const R *u, const R *delta)
+    {
+        bool ok = true;
+        R S[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) S[n] = R(0);
+        size = R(0);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const R cj = R(Lattice<DIM>::sign(k)) * P.c[Lattice<DIM>::axis(k)] * P.inv2V;
+            const R D = R(1) / R(Q) + cj * u[0];
+            ok &= D > R(0);
+            const R dr = delta[k] * rcp_fast(D);
+            a[k] = delta[k] * dr;
+            y[k] = R(-0.5) * cj * (dr * rcp_fast(D));
+            ok &= fabs(y[k]) <= most_rough;
+            size = fmax(size, fabs(y[k]));
+            R p = a[k];
+            S[0] += p;
+#pragma unroll
+            for (int n = 1; n < N; ++n) {
+                p *= y[k];
+                S[n] += p;
+            }
+        }
+        constexpr double cat[8] = {1.0 / 2, 1.0 / 3, 2.0 / 4, 5.0 / 5, 14.0 / 6, 42.0 / 7, 132.0 / 8, 429.0 / 9};
+#pragma unroll
+        for (int n = 0; n < N; ++n) c[n] = R(cat[n]) * S[n];
+        return ok;
+    }
+
+    // B(t) and dB/dt
+    __host__ __device__ __forceinline__ bool eval(R t, R &B, R &dB) const
+    {
+        R b = R(0), db = R(0);
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const R X = R(1) - R(4) * y[k] * t;
+            ok &= X > R(0);
+            const R s = sqrt_fast(X);
+            const R q = rcp_fast(R(1) + s);
+            const R aq = a[k] * q;
+            db += aq;
+            b += aq * (q * (R(1) + R(2) * s));
+        }
+        B = b * (t * t) * R(2.0 / 3.0);
+        dB = db * (R(2) * t);
+        return ok;
+    }
+};
+
+template <int DIM, class R> struct Expansion<ShallowWater<DIM>, R> {
+    static constexpr int Q = Lattice<DIM>::Q, M = DIM + 1;
+    static constexpr int N = 4;
+    // sizes measured as above: at most, the error is 2e-7 (FP32) and 1e-16 (FP64); three times that size
+    // multiplies it by 3^5
+    static constexpr int STEPS = sizeof(R) == 4 ? 0 : 1;
+    static constexpr R most = sizeof(R) == 4 ? R(0.02) : R(3e-4);
+    static constexpr R most_rough = R(2);
+    R c[N], size;
+    R kap[Q], cv[Q], eta[Q], rr[Q], w[Q], zt[Q], z1[Q], z2[Q];
+
+    __host__ __device__ __forceinline__ bool build(const ParamsR<R> &P, const R *u, const R *delta)
+    {
+        bool ok = u[0] > R(0);
+        const R rh = rcp_fast(u[0]);
+        const R rf = R(2) * P.V * rh;          // 1 / f_1 = rf / c
+        const R gh2 = R(0.5) * P.g * u[0];
+        const R hV = u[0] * P.inv2V;
+        const R nu = R(2) * P.V / R(Q);
+        R v[DIM];
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) v[j] = u[1 + j] * rh;
+#pragma unroll
+        for (int n = 0; n < N; ++n) c[n] = R(0);
+        size = R(0);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const int d = Lattice<DIM>::axis(k);
+            const R sg = R(Lattice<DIM>::sign(k));
+            const R ck = nu + sg * v[d];
+            const R rc = rcp_fast(ck);
+            const R rc2 = rc * rc;
+            const R kp = gh2 * rc2;
+            const R curv = R(1) - R(2) * kp;
+            ok &= (ck > R(0)) & (curv > R(0));
+            const R L = rcp_fast(curv);
+            const R e1 = delta[k * M] * (rf * rc);
+            const R R1 = (sg * rf * rc2) * (delta[k * M + 1 + d] - v[d] * delta[k * M]);
+            const R A = (e1 - R1) * L;
+            const R b1 = A - e1;
+            const R wk = hV * ck * (ck * ck);
+            const R A2 = A * A, Ab = A * b1, b11 = b1 * b1;
+            const R n2 = kp * (R(2) * Ab + A2) - e1 * b1;  // (1 - 2 kappa) beta_2
+            const R b2 = n2 * L;
+            const R kA2 = kp * A2;
+            const R sz = L * (fabs(e1 + R1) + R(6) * kp * fabs(A)) + fabs(A) + fabs(e1);
+            ok &= sz <= most_rough;
+            size = fmax(size, sz);
+            c[0] += wk * (kp * (e1 * e1) + R(0.5) * curv * b11);
+            c[1] += wk * (kA2 * b1 - R(0.5) * e1 * b11);
+            c[2] += wk * (R(0.5) * b2 * n2 + kA2 * b11);
+            c[3] += wk * (kp * (b2 * (b2 * (b1 + R(2) * A) + R(2) * Ab * (b1 + A)) + A2 * b11 * b1) -
+                          R(0.5) * e1 * (b2 * b2));
+            if constexpr (DIM == 2) {
+                const R tau = delta[k * M + 2 - d] - v[1 - d] * delta[k * M];
+                R z = R(0.5) * tau * tau * (rf * rc);
+                zt[k] = z;
+                c[0] += z;
+                z *= -e1;
+                c[1] += z;
+                z *= -e1;
+                c[2] += z;
+                c[3] -= z * e1;
+            }
+            kap[k] = kp;
+            cv[k] = curv;
+            eta[k] = e1;
+            rr[k] = R1;
+            w[k] = wk;
+            z1[k] = A;
+            z2[k] = b2 + b1 * A;
+        }
+        return ok;
+    }
+
+    // B(t) and dB/dt.  z = (eta + beta) / (1 - beta) solves kappa z^3 + 3 kappa z^2 - k1 z + k0 = 0 (Newton from
+    // the expansion, the populations in step); with R eliminated by the stationarity of Psi,
+    //   Psi = kappa [(eta + z beta)^2 - 2 z^2 beta] + ((1 + eta) / 2 - kappa) beta^2
+    // has no cancellation at leading order.
+    __host__ __device__ __forceinline__ bool eval(R t, R &B, R &dB) const
+    {
+        constexpr R tol = R(sizeof(R) == 4 ? 1e-4 : 1e-9);
+        R z[Q], k0[Q], k1[Q];
+        bool ok = true, more = true;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const R et = t * eta[k];
+            k1[k] = cv[k] + t * (eta[k] + rr[k]);
+            k0[k] = t * (eta[k] - rr[k]) + et * et;
+            z[k] = t * (z1[k] + t * z2[k]);
+        }
+        for (int it = 0; it < 6 && more; ++it) {
+            more = false;
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                const R g = k0[k] + z[k] * (kap[k] * z[k] * (R(3) + z[k]) - k1[k]);
+                const R gp = R(3) * kap[k] * z[k] * (R(2) + z[k]) - k1[k];
+                ok &= gp < R(0);
+                const R dz = g * rcp_fast(gp);
+                z[k] -= dz;
+                more |= !(fabs(dz) <= tol * fabs(z[k]));
+            }
+        }
+        ok &= !more;
+        R b = R(0), db = R(0);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const R et = t * eta[k], m = R(1) + et;
+            const R q = R(1) + z[k];
+            ok &= (m > R(0)) & (q > R(0));
+            const R be = (z[k] - et) * rcp_fast(q);
+            const R b2 = be * be, x = et + z[k] * be;
+            b += w[k] * (kap[k] * (x * x - R(2) * z[k] * z[k] * be) + R(0.5) * (cv[k] + et) * b2);
+            db += w[k] * ((R(2) * kap[k] * z[k] - R(0.5) * b2) * eta[k] - be * rr[k]);
+            if constexpr (DIM == 2) {
+                const R rm = rcp_fast(m), q2 = zt[k] * t * rm;
+                b += q2 * t;
+                db += q2 * (R(1) + rm);
+            }
+        }
+        B = b;
+        dB = db;
+        return ok;
+    }
+};
+
+// Cells too rough for the truncated expansion: Newton on B(t) - B(-1) from its root; then the general search.
+template <class Sys, class R>
+__host__ __device__ __forceinline__ bool rough_root(const ParamsR<R> &P, const R *u, const R *delta, R &omega)
+{
+    Expansion<Sys, R> X;
+    if (!X.build(P, u, delta)) return false;
+    R E0, dE0;
+    if (!X.eval(R(-1), E0, dE0) || !(E0 > R(0))) return false;
+    R t = R(1) + expansion_root<R, Expansion<Sys, R>::N>(X.c, 0);
+    if (!(t > R(0.25) && t < R(2))) t = R(1);
+    constexpr R tol = R(sizeof(R) == 4 ? 1e-4 : 1e-9);
+    R dt = R(1), dB = R(1);
+    for (int it = 0; it < 8; ++it) {
+        R B;
+        if (!X.eval(t, B, dB) || !(dB > R(0))) return false;
+        dt = (B - E0) * rcp_fast(dB);
+        t -= dt;
+        if (!(t > R(0.1) && t < R(2.5))) return false;
+        if (fabs(dt) <= tol) break;
+    }
+    if (!(fabs(dt) <= tol && t < P.t_max)) return false;
+    // (the Newton point of a convex F lies above its root by less than dt^2, below the rounding of omega)
+    omega = R(1) + t;
+    return true;
+}
+
+// omega of a cell that the truncated expansion does not certify; out of line, so that its registers do
+// not add to those of the kernels' common path
+template <class Sys, class R>
+__device__ __noinline__ R rough_omega(const ParamsR<R> &P, const R *u, const R *delta, bool &fallback)
+{
+    R w;
+    if (rough_root<Sys, R>(P, u, delta, w)) {
+        fallback = false;
+        return w;
+    }
+    typename Sys::template Ctx<R> cx;
+    Sys::template prepare<R>(P, u, delta, cx);
+    return entropic_omega<Sys, R>(P, cx, fallback);
+}
+
+// omega = 1 + t* (no root: 1, and fallback is set)
+template <class Sys, class R>
+__device__ __forceinline__ R omega_of(const ParamsR<R> &P, const R *u, const R *delta, bool &fallback)
+{
+    using X = Expansion<Sys, R>;
+    X x;
+    if (x.build(P, u, delta) && x.size <= X::most) {
+        // |e| <= 4 size: below a quarter of the last place omega is 2 (and c_2 may have underflowed)
+        const R e = x.size <= Eps<R>::value / R(16) ? R(0) : expansion_root<R, X::N>(x.c, X::STEPS);
+        if (R(1) + e < P.t_max) {
+            fallback = false;
+            return R(2) + e;
+        }
+    }
+    R uu[Sys::M], dd[Sys::Q * Sys::M];
+#pragma unroll
+    for (int m = 0; m < Sys::M; ++m) uu[m] = u[m];
+#pragma unroll
+    for (int i = 0; i < Sys::Q * Sys::M; ++i) dd[i] = delta[i];
+    bool fb = false;
+    const R w = rough_omega<Sys, R>(P, uu, dd, fb);
+    fallback = fb;
+    return w;
+}
+
+}  // namespace eslbm

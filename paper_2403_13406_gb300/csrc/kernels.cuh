@@ -9,7 +9,7 @@
 
 #include <cooperative_groups.h>
 
-#include "systems.cuh"
+#include "expansion.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -19,6 +19,17 @@ constexpr int kBlock = 256;       // threads per block of the per-cell kernels
 constexpr int kFusedBlock = 256;  // threads per block of the temporally blocked 1D kernel
 constexpr int kRedBlocks = 1024;  // fixed grid of the totals reduction (deterministic order)
 constexpr int kRedThreads = 256;
+
+// Resident blocks of kBlock threads per SM that the relaxation's registers are held to.  The entropic
+// relaxations' out-of-line root-find of rough cells would otherwise set the registers of the whole kernel
+// (FP32 shallow water: 176, one block per SM; its common path needs 64 to 80).
+template <class Sys, class R, int OM> constexpr int relax_min_blocks()
+{
+    if (OM == OM_FIXED || Sys::LINEAR) return 1;
+    if (sizeof(R) == 8) return Sys::M == 1 ? 2 : 1;
+    if (OM == OM_MIXED) return 2;
+    return Sys::M == 1 ? 4 : 3;
+}
 
 template <class R> struct StageArgs {
     const R *__restrict__ fin;
@@ -172,6 +183,23 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
         for (int m = 0; m < M; ++m) ud[m] = double(u[m]);
 #pragma unroll
         for (int i = 0; i < Q * M; ++i) dd[i] = double(delta[i]);
+        // Where the FP64 root 1 + wd is at hand, F(t) <= 0 up to it.  The kernel's FP32 constants 4 g V and
+        // 1 / (16 g V) are rounded on their own, which moves the root of the F they define by about 2^-23 of
+        // the size of a population's odd terms: stay a few times that below.
+        using X = Expansion<Sys, double>;
+        X x;
+        double wd = 0.0;
+        bool found = false;
+        if (x.build(Pd, ud, dd) && x.size <= X::most) {
+            wd = x.size <= Eps<double>::value / 16.0 ? 2.0 : 2.0 + expansion_root<double, X::N>(x.c, X::STEPS);
+            found = wd < 1.0 + Pd.t_max;
+        } else {
+            found = rough_root<Sys, double>(Pd, ud, dd, wd);
+        }
+        if (found) {
+            wd -= x.size * 0x1p-20;
+            return double(w) <= wd ? w : __double2float_rz(wd);
+        }
         typename Sys::template Ctx<double> cx;
         Sys::template prepare<double>(Pd, ud, dd, cx);
         double E0, dE0, Bt, dBt;
@@ -218,9 +246,7 @@ __device__ __forceinline__ void relax_cell(const ParamsR<R> &P, R *f, int kind, 
     }
     R w = P.omega;
     if constexpr (OM != OM_FIXED && !Sys::LINEAR) {
-        typename Sys::template Ctx<R> cx;
-        Sys::template prepare<R>(P, u, delta, cx);
-        w = entropic_omega<Sys, R>(P, cx, fallback);
+        w = omega_of<Sys, R>(P, u, delta, fallback);
         if constexpr (OM == OM_MIXED) w = mixed_omega<Sys, R>(P, u, delta, w, fallback);
     } else if constexpr (OM != OM_FIXED) {
         w = R(2);  // quadratic kinetic entropies: omega* = 2 exactly (Proposition 2)
@@ -244,7 +270,7 @@ __device__ __forceinline__ R *record_of(const ParamsR<R> &P, int st, int64_t cel
 
 // Fused stage: pull-shift by sh (transport, eq. transportPhase) then relax.
 template <class Sys, int DIM, class R, int OM>
-__global__ void __launch_bounds__(kBlock) k_stage(StageArgs<R> a, ParamsR<R> P)
+__global__ void __launch_bounds__(kBlock, relax_min_blocks<Sys, R, OM>()) k_stage(StageArgs<R> a, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -302,7 +328,7 @@ template <class R> struct BulkArgs {
 };
 
 template <class Sys, class R, int OM>
-__global__ void __launch_bounds__(kRowThreads) k_stage_bulk(BulkArgs<R> a, ParamsR<R> P)
+__global__ void __launch_bounds__(kRowThreads, relax_min_blocks<Sys, R, OM>()) k_stage_bulk(BulkArgs<R> a, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M, NP = Q * M;
     constexpr int V4 = 16 / (int)sizeof(R);  // elements per 16 bytes
@@ -426,7 +452,7 @@ template <class R, int OM> constexpr int step1d_min_blocks() { return (sizeof(R)
 
 template <class Sys, class R, int OM, bool RECORD = false>
 __global__ void __launch_bounds__(kFusedBlock, step1d_min_blocks<R, OM>())
-    k_step1d(FusedArgs<R> a, StageList sl, ParamsR<R> P)
+    k_step1d(FusedArgs<R> a, StageList sl, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M, NP = Q * M;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -558,14 +584,14 @@ __device__ __forceinline__ void relax_adjoint(const ParamsR<R> &P, const R *f, c
     R w = P.omega;
     bool varying = false;
     typename Sys::template Ctx<R> cx;
-    R Dm[Q * M];  // dual deviations at t = -1, from the root-find's own evaluation there
+    R Dm[Q * M];  // dual deviations at t = -1
     if constexpr (OM != OM_FIXED && !Sys::LINEAR) {
-        Sys::template prepare<R>(P, u, delta, cx);
         bool fb = false;
-        R E0 = R(0);
-        w = entropic_omega<Sys, R>(P, cx, fb, Dm, &E0);
+        w = omega_of<Sys, R>(P, u, delta, fb);
         if constexpr (OM == OM_MIXED) w = mixed_omega<Sys, R>(P, u, delta, w, fb);
-        varying = !fb && E0 > R(0);
+        Sys::template prepare<R>(P, u, delta, cx);
+        R E0, dE0;
+        varying = Sys::template eval<R>(P, cx, R(-1), E0, dE0, Dm) && !fb && E0 > R(0);
     } else if constexpr (OM != OM_FIXED) {
         w = R(2);
     }
@@ -609,7 +635,7 @@ __device__ __forceinline__ void relax_adjoint(const ParamsR<R> &P, const R *f, c
 template <class Sys, int DIM, class R, int OM>
 __global__ void __launch_bounds__(kBlock) k_adjoint_stage(const R *__restrict__ fin, const R *__restrict__ gout,
                                                           R *__restrict__ gin, int64_t nx, int64_t ny, Shift sh,
-                                                          int kind, ParamsR<R> P)
+                                                          int kind, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -655,7 +681,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_readout(const double *__rest
 // dJ/du0 = sum_k E_k(u0)^T g_k for f_0 = f^eq(u0)
 template <class Sys, class R>
 __global__ void __launch_bounds__(kBlock) k_adjoint_init(const double *__restrict__ u0, const R *__restrict__ g,
-                                                         double *__restrict__ du0, int64_t ncell, ParamsR<R> P)
+                                                         double *__restrict__ du0, int64_t ncell, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -699,7 +725,7 @@ template <class R> struct BatchArgs {
 };
 
 template <class Sys, class R, int OM>
-__global__ void __launch_bounds__(kBlock) k_batch_step(BatchArgs<R> a, StageList sl, ParamsR<R> P)
+__global__ void __launch_bounds__(kBlock, relax_min_blocks<Sys, R, OM>()) k_batch_step(BatchArgs<R> a, StageList sl, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     cg::grid_group grid = cg::this_grid();
@@ -764,7 +790,7 @@ template <class R> struct BatchAdjointArgs {
 };
 
 template <class Sys, class R, int OM>
-__global__ void __launch_bounds__(kBlock) k_batch_adjoint_step(BatchAdjointArgs<R> a, StageList sl, ParamsR<R> P)
+__global__ void __launch_bounds__(kBlock) k_batch_adjoint_step(BatchAdjointArgs<R> a, StageList sl, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     cg::grid_group grid = cg::this_grid();
@@ -813,7 +839,7 @@ __global__ void __launch_bounds__(kBlock) k_batch_adjoint_step(BatchAdjointArgs<
 // f_k = f^eq_k(u0) (Section 3.1) with the domain check of Section 1.2.
 template <class Sys, class R>
 __global__ void __launch_bounds__(kBlock) k_init_eq(const double *__restrict__ u0, R *__restrict__ f,
-                                                    int64_t ncell, ParamsR<double> P, Counters *cnt)
+                                                    int64_t ncell, const __grid_constant__ ParamsR<double> P, Counters *cnt)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -907,7 +933,7 @@ __device__ __forceinline__ double block_sum(double v, double *part)
 // set of cells in a fixed tree order into partials[block][2 + M].
 template <class Sys, int DIM, class R>
 __global__ void __launch_bounds__(kRedThreads) k_totals_partial(const R *__restrict__ f, double *__restrict__ partials,
-                                                                int64_t nx, int64_t ny, Shift sh, ParamsR<double> P)
+                                                                int64_t nx, int64_t ny, Shift sh, const __grid_constant__ ParamsR<double> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M, NV = 2 + M;
     const int64_t ncell = nx * ny;

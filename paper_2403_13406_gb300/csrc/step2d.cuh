@@ -64,7 +64,7 @@ template <class Sys, class R, int OM> struct Step2dThreads {
 
 template <class Sys, class R, int OM>
 __global__ void __launch_bounds__(Step2dThreads<Sys, R, OM>::value, kStep2dBlocksPerSm)
-    k_step2d(Step2dArgs<R> a, StageList sl, ParamsR<R> P)
+    k_step2d(Step2dArgs<R> a, StageList sl, const __grid_constant__ ParamsR<R> P)
 {
     constexpr int Q = Sys::Q, M = Sys::M, NP = Q * M;
     static_assert(Q == 4, "D2Q4 only");
