@@ -73,7 +73,13 @@ static cudaError_t gather_t(const void *f, double *out, int64_t nx, int64_t ny, 
                             const Shift &sh, const double *fbar, cudaStream_t st)
 {
     RefPlanes ref;
-    for (int i = 0; i < 16; ++i) ref.fbar[i] = fbar ? fbar[i] : 0.0;
+    ref.shifted = 0;
+    for (int m = 0; m < 4; ++m) ref.ubar[m] = 0.0;
+    for (int i = 0; i < 16; ++i) {
+        ref.fbar[i] = fbar ? fbar[i] : 0.0;
+        ref.shifted |= ref.fbar[i] != 0.0;
+        if (i < 2 * DIM * M) ref.ubar[i % M] += ref.fbar[i];
+    }
     dim3 grid((unsigned)((nx + kBlock - 1) / kBlock), (unsigned)ny);
     k_gather<DIM, R, MOM><<<grid, kBlock, 0, st>>>((const R *)f, out, nx, ny, M, p0, np, sh, ref);
     return cudaGetLastError();

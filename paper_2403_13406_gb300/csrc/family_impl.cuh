@@ -307,8 +307,9 @@ cudaError_t init_family(bool fp64, const double *u0, void *f, int64_t ncell, con
 {
     const unsigned grid = (unsigned)((ncell + kBlock - 1) / kBlock);
     const ParamsR<double> Pd = params_as<double>(P);
-    if (fp64) k_init_eq<Sys, double><<<grid, kBlock, 0, st>>>(u0, (double *)f, ncell, Pd, cnt);
-    else k_init_eq<Sys, float><<<grid, kBlock, 0, st>>>(u0, (float *)f, ncell, Pd, cnt);
+    const ParamsR<dfloat> Pp = params_as<dfloat>(P);
+    if (fp64) k_init_eq<Sys, double><<<grid, kBlock, 0, st>>>(u0, (double *)f, ncell, Pd, Pp, cnt);
+    else k_init_eq<Sys, float><<<grid, kBlock, 0, st>>>(u0, (float *)f, ncell, Pd, Pp, cnt);
     return cudaGetLastError();
 }
 

@@ -9,6 +9,7 @@
 
 #include <cooperative_groups.h>
 
+#include "dfloat.cuh"
 #include "expansion.cuh"
 
 namespace cg = cooperative_groups;
@@ -861,10 +862,30 @@ __global__ void __launch_bounds__(kBlock) k_batch_adjoint_step(BatchAdjointArgs<
     }
 }
 
-// f_k = f^eq_k(u0) (Section 3.1) with the domain check of Section 1.2.
+// f_k = f^eq_k(u0) (Section 3.1) with the domain check of Section 1.2, in 64 bits.
+template <class Sys, class R>
+__device__ __forceinline__ void init_cell(const ParamsR<double> &P, const double *u, R *f, bool &bad)
+{
+    constexpr int NP = Sys::Q * Sys::M;
+    bad = !Sys::template admissible<double>(P, u);
+    double feq[NP];
+    Sys::template equilibrium<double>(P, u, feq);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) f[j] = R(P.shifted ? feq[j] - P.fbar[j] : feq[j]);
+}
+template <class Sys, class R>
+__device__ __noinline__ void init_cell_general(const ParamsR<double> &P, const double *u, R *f, bool &bad)
+{
+    init_cell<Sys, R>(P, u, f, bad);
+}
+
+// FP32 lattices: the equilibrium in pairs of FP32 numbers (dfloat.cuh) rounded to FP32 at the end, where the
+// fields are of ordinary size and an FP32 test finds them inside the domain by a margin far above its
+// rounding; other cells in FP64.
 template <class Sys, class R>
 __global__ void __launch_bounds__(kBlock) k_init_eq(const double *__restrict__ u0, R *__restrict__ f,
-                                                    int64_t ncell, const __grid_constant__ ParamsR<double> P, Counters *cnt)
+                                                    int64_t ncell, const __grid_constant__ ParamsR<double> P,
+                                                    const __grid_constant__ ParamsR<dfloat> Pp, Counters *cnt)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -876,11 +897,37 @@ __global__ void __launch_bounds__(kBlock) k_init_eq(const double *__restrict__ u
             u[m] = u0[(int64_t)m * ncell + i];
             nonfinite |= !isfinite(u[m]);
         }
-        bad = !Sys::template admissible<double>(P, u);
-        double feq[Q * M];
-        Sys::template equilibrium<double>(P, u, feq);
+        R out[Q * M];
+        if constexpr (sizeof(R) == 4) {
+            dfloat up[M];
+            float uf[M];
+            bool ok = true;
 #pragma unroll
-        for (int j = 0; j < Q * M; ++j) f[(int64_t)j * ncell + i] = R(P.shifted ? feq[j] - P.fbar[j] : feq[j]);
+            for (int m = 0; m < M; ++m) {
+                ok &= to_pair(u[m], up[m]);
+                uf[m] = up[m].hi;
+            }
+            if (ok && Sys::well_inside(Pp, uf)) {
+                dfloat feq[Q * M];
+                Sys::template equilibrium<dfloat>(Pp, up, feq);
+#pragma unroll
+                for (int j = 0; j < Q * M; ++j) out[j] = P.shifted ? (feq[j] - Pp.fbar[j]).hi : feq[j].hi;
+            } else {
+                double uu[M];
+#pragma unroll
+                for (int m = 0; m < M; ++m) uu[m] = u[m];
+                R oo[Q * M];
+                bool b = false;
+                init_cell_general<Sys, R>(P, uu, oo, b);
+                bad = b;
+#pragma unroll
+                for (int j = 0; j < Q * M; ++j) out[j] = oo[j];
+            }
+        } else {
+            init_cell<Sys, R>(P, u, out, bad);
+        }
+#pragma unroll
+        for (int j = 0; j < Q * M; ++j) f[(int64_t)j * ncell + i] = out[j];
     }
     warp_count(bad, &cnt->domain_violations);
     warp_count(nonfinite, &cnt->non_finite);
@@ -906,6 +953,8 @@ __global__ void __launch_bounds__(kBlock) k_set(const double *__restrict__ src, 
 // shifted storage f = stored + fbar).
 struct RefPlanes {
     double fbar[16];
+    double ubar[4];  // sum_k fbar_k (exact: a few values of the storage precision)
+    int shifted;     // whether any of them is not zero
 };
 
 template <int DIM, class R, bool MOMENTS>
@@ -918,11 +967,21 @@ __global__ void __launch_bounds__(kBlock) k_gather(const R *__restrict__ f, doub
     if (x >= nx) return;
     const int64_t ncell = nx * ny, o = y * nx + x;
     if (MOMENTS) {
+        int64_t src[Q];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) src[k] = src_cell<DIM>(k, x, y, nx, ny, sh);
         for (int m = 0; m < M; ++m) {
             double s = 0.0;
+            if constexpr (sizeof(R) == 4) {
+                R v[Q];
 #pragma unroll
-            for (int k = 0; k < Q; ++k)
-                s += double(f[(int64_t)(k * M + m) * ncell + src_cell<DIM>(k, x, y, nx, ny, sh)]) + ref.fbar[k * M + m];
+                for (int k = 0; k < Q; ++k) v[k] = f[(int64_t)(k * M + m) * ncell + src[k]];
+                s = sum_exact<Q>(v);
+                if (ref.shifted) s += ref.ubar[m];
+            } else {
+#pragma unroll
+                for (int k = 0; k < Q; ++k) s += f[(int64_t)(k * M + m) * ncell + src[k]] + ref.fbar[k * M + m];
+            }
             out[(int64_t)m * ncell + o] = s;
         }
     } else {

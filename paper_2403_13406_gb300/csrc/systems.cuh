@@ -134,6 +134,18 @@ template <int DIM, bool BURGERS> struct Scalar {
         return isfinite(u[0]);
     }
 
+    // admissible by a margin of 1e-4, evaluated in FP32 (rounding: a few 1e-7)
+    template <class PP> __device__ static bool well_inside(const PP &P, const float *u)
+    {
+        bool ok = true;
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) {
+            const float slope = BURGERS ? P.c[j].hi * u[0] : P.a[j].hi;
+            ok &= fabsf(slope) * float(Q) < 1.9998f * P.V.hi;
+        }
+        return ok;
+    }
+
     template <class R> __device__ static R entropy(const ParamsR<R> &, const R *u) { return R(0.5) * u[0] * u[0]; }
 
     template <class R> struct Ctx {
@@ -305,6 +317,17 @@ template <int DIM> struct ShallowWater {
             if (!(fabs(v) + cs < nu)) return false;
         }
         return true;
+    }
+
+    // admissible by a margin of 1e-4, evaluated in FP32 (rounding: a few 1e-7)
+    template <class PP> __device__ static bool well_inside(const PP &P, const float *u)
+    {
+        const float h = u[0];
+        bool ok = h > 0.0f;
+        const float cs = sqrtf(P.g.hi * h), rh = __fdividef(1.0f, h);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) ok &= (fabsf(u[1 + j] * rh) + cs) * float(Q) < 1.9998f * P.V.hi;
+        return ok;
     }
 
     template <class R> __device__ static R entropy(const ParamsR<R> &P, const R *u)
@@ -577,6 +600,13 @@ struct Euler2 {
         if (!(rho > R(0))) return false;
         const R p = P.gamma_m1 * (u[3] - R(0.5) * (u[1] * u[1] + u[2] * u[2]) / rho);
         return p > R(0) && isfinite(p);
+    }
+
+    // admissible by a margin of 1e-4 of the energy, evaluated in FP32 (rounding: a few 1e-7 of it)
+    template <class PP> __device__ static bool well_inside(const PP &P, const float *u)
+    {
+        const float e = u[3] - 0.5f * (u[1] * u[1] + u[2] * u[2]) * __fdividef(1.0f, u[0]);
+        return u[0] > 0.0f && P.gamma_m1.hi > 0.0f && e > 1e-4f * fabsf(u[3]) && u[3] < 1e30f;
     }
 
     template <class R> __device__ static R entropy(const ParamsR<R> &, const R *) { return R(NAN); }
