@@ -32,7 +32,8 @@
 // and SM, in FP64).  Two evaluations of B by inner Newton solves, a quartic model through them and its
 // certificate took 652 thread instructions per 1D shallow-water cell-stage in all; with the expansion 305.
 // Before -> after: 1D shallow water N = 2^20, FP32, 409 -> 186 us per step; 2D Burgers 4096^2, FP32, 296 -> 141 us
-// per stage; 1D shallow water N = 100003, FP64, 3.26 -> 0.82 ms per step.
+// per stage; 1D shallow water N = 100003, FP64, 3.26 -> 0.82 ms per step.  With the populations in packed pairs and
+// two coefficients for very smooth cells (SmoothRoot) 139 us per step and 110 us per stage (FP32).
 #pragma once
 
 #include "systems.cuh"
@@ -318,6 +319,195 @@ template <int DIM, class R> struct Expansion<ShallowWater<DIM>, R> {
     }
 };
 
+// Two values, one for each of a pair of opposite populations (k and k + Q/2): on the device pairs of FP32
+// are the packed operands of one instruction, so the common path issues half as many.
+template <class R> struct Two {
+    R x, y;
+};
+template <class R> __host__ __device__ __forceinline__ Two<R> two(R x, R y) { return {x, y}; }
+template <class R> __host__ __device__ __forceinline__ Two<R> two(R x) { return {x, x}; }
+template <class R> __host__ __device__ __forceinline__ Two<R> fma2(const Two<R> &a, const Two<R> &b, const Two<R> &c)
+{
+#ifdef __CUDA_ARCH__
+    if constexpr (sizeof(R) == 4) {
+        const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
+        return {r.x, r.y};
+    }
+#endif
+    return {fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
+}
+template <class R> __host__ __device__ __forceinline__ Two<R> operator*(const Two<R> &a, const Two<R> &b)
+{
+#ifdef __CUDA_ARCH__
+    if constexpr (sizeof(R) == 4) {
+        const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+        return {r.x, r.y};
+    }
+#endif
+    return {a.x * b.x, a.y * b.y};
+}
+template <class R> __host__ __device__ __forceinline__ Two<R> operator+(const Two<R> &a, const Two<R> &b)
+{
+#ifdef __CUDA_ARCH__
+    if constexpr (sizeof(R) == 4) {
+        const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+        return {r.x, r.y};
+    }
+#endif
+    return {a.x + b.x, a.y + b.y};
+}
+template <class R> __host__ __device__ __forceinline__ Two<R> rcp2(const Two<R> &a) { return {rcp_fast(a.x), rcp_fast(a.y)}; }
+
+// SmoothRoot<Sys, R>::find: the root e of a smooth cell from the expansion (the terms of Expansion, in pairs of
+// populations); false where the cell is too rough for it or outside the domain.  Its measure of roughness is
+// the sum of squares sq of the terms' ratios.  Very smooth cells (FP32, up to `few`: the terms of order
+// size^3 in omega are below its rounding) need c_2 and c_3 only: e = -c_3 / (c_2 + c_3).  Worst error of omega on the
+// random cells above: FP32 scalar 4e-8 up to `few` and up to `most`, shallow water 5e-8 up to `few`, 1e-6 up to
+// `most` (next to the domain's edge; what Newton on the closed form gives there too), FP64 6e-17.
+template <class Sys, class R> struct SmoothRoot;
+
+template <int DIM, class R> struct SmoothRoot<Scalar<DIM, true>, R> {
+    static constexpr int Q = Lattice<DIM>::Q;
+    static constexpr int N = Expansion<Scalar<DIM, true>, R>::N;
+    static constexpr R few = sizeof(R) == 4 ? R(2.5e-3) : R(0);
+    static constexpr R most = sizeof(R) == 4 ? R(0.04) : R(0.004);
+
+    __host__ __device__ static __forceinline__ bool find(const ParamsR<R> &P, const R *u, const R *delta, R &e)
+    {
+        Two<R> S0 = two(R(0)), S1 = two(R(0)), sq = two(R(0)), y[Q / 2], p[Q / 2];
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < Q / 2; ++k) {
+            const R cj = P.c[Lattice<DIM>::axis(k)] * P.inv2V;
+            const R s = cj * u[0];
+            ok &= fabs(s) < R(1) / R(Q);
+            const Two<R> rD = rcp2(two(R(1) / R(Q) + s, R(1) / R(Q) - s));
+            const Two<R> d = two(delta[k], delta[k + Q / 2]);
+            const Two<R> dr = d * rD, a = d * dr;
+            y[k] = dr * (rD * two(R(-0.5) * cj, R(0.5) * cj));
+            sq = fma2(y[k], y[k], sq);
+            p[k] = a * y[k];
+            S0 = S0 + a;
+            S1 = S1 + p[k];
+        }
+        const R q = sq.x + sq.y;
+        if (!(ok && q <= most * most)) return false;
+        constexpr R tiny = Eps<R>::value / R(16);
+        const R s0 = S0.x + S0.y, s1 = S1.x + S1.y;
+        if (sizeof(R) == 4 && q <= few * few) {
+            const R c3 = s1 * R(2.0 / 3.0);  // over c_2 = s0 / 2
+            e = q <= tiny * tiny ? R(0) : -c3 * rcp_fast(s0 + c3);
+            return true;
+        }
+        if (q <= tiny * tiny) {
+            e = R(0);
+            return true;
+        }
+        constexpr double cat[8] = {1.0 / 2, 1.0 / 3, 2.0 / 4, 5.0 / 5, 14.0 / 6, 42.0 / 7, 132.0 / 8, 429.0 / 9};
+        R c[N];
+        c[0] = R(cat[0]) * s0;
+        c[1] = R(cat[1]) * s1;
+#pragma unroll
+        for (int n = 2; n < N; ++n) {
+            Two<R> S = two(R(0));
+#pragma unroll
+            for (int k = 0; k < Q / 2; ++k) {
+                p[k] = p[k] * y[k];
+                S = S + p[k];
+            }
+            c[n] = R(cat[n]) * (S.x + S.y);
+        }
+        e = expansion_root<R, N>(c, sizeof(R) == 4 ? 0 : 1);
+        return true;
+    }
+};
+
+template <int DIM, class R> struct SmoothRoot<ShallowWater<DIM>, R> {
+    static constexpr int Q = Lattice<DIM>::Q, M = DIM + 1;
+    static constexpr R few = sizeof(R) == 4 ? R(2e-3) : R(0);
+    static constexpr R most = sizeof(R) == 4 ? R(0.02) : R(3e-4);
+
+    __host__ __device__ static __forceinline__ bool find(const ParamsR<R> &P, const R *u, const R *delta, R &e)
+    {
+        const R rh = rcp_fast(u[0]);
+        const R rf = R(2) * P.V * rh;  // 1 / f_1 = rf / c
+        const R gh = P.g * u[0], gh2 = R(0.5) * gh;
+        const R hV = u[0] * P.inv2V;
+        const R nu = R(2) * P.V / R(Q);
+        bool ok = u[0] > R(0);
+        Two<R> C2 = two(R(0)), C3 = two(R(0)), sq = two(R(0));
+        Two<R> kp[Q / 2], e1[Q / 2], A[Q / 2], b1[Q / 2], w[Q / 2], L[Q / 2], zt[Q / 2];
+#pragma unroll
+        for (int k = 0; k < Q / 2; ++k) {
+            constexpr int H = Q / 2;
+            const int d = Lattice<DIM>::axis(k);
+            const R v = u[1 + d] * rh;
+            const R t = nu - fabs(v);  // min c
+            ok &= (t > R(0)) & (t * t > gh);
+            const Two<R> c = two(nu + v, nu - v);
+            const Two<R> rc = rcp2(c), rc2 = rc * rc;
+            kp[k] = two(gh2) * rc2;
+            const Two<R> cv = fma2(two(R(-2)), kp[k], two(R(1)));
+            L[k] = rcp2(cv);
+            const Two<R> d0 = two(delta[k * M], delta[(k + H) * M]);
+            const Two<R> d1 = two(delta[k * M + 1 + d], delta[(k + H) * M + 1 + d]);
+            const Two<R> frc = two(rf) * rc;
+            e1[k] = d0 * frc;
+            const Two<R> r1 = (rc2 * two(rf, -rf)) * fma2(two(-v), d0, d1);
+            A[k] = fma2(two(R(-1)), r1, e1[k]) * L[k];
+            b1[k] = fma2(two(R(-1)), e1[k], A[k]);
+            w[k] = (two(hV) * c) * (c * c);
+            const Two<R> e11 = e1[k] * e1[k], A2 = A[k] * A[k], b11 = b1[k] * b1[k];
+            sq = fma2(L[k] * L[k], e11 + A2, sq);
+            C2 = fma2(w[k], fma2(kp[k], e11, (two(R(0.5)) * cv) * b11), C2);
+            C3 = fma2(w[k], fma2(kp[k] * A2, b1[k], (two(R(-0.5)) * e1[k]) * b11), C3);
+            if constexpr (DIM == 2) {
+                const R vt = u[2 - d] * rh;
+                const Two<R> d2 = two(delta[k * M + 2 - d], delta[(k + H) * M + 2 - d]);
+                const Two<R> tau = fma2(two(-vt), d0, d2);
+                const Two<R> z = (two(R(0.5)) * frc) * (tau * tau);
+                zt[k] = z * e1[k];
+                C2 = C2 + z;
+                C3 = fma2(two(R(-1)), zt[k], C3);
+            }
+        }
+        const R q = sq.x + sq.y;
+        if (!(ok && q <= most * most)) return false;
+        constexpr R tiny = Eps<R>::value / R(64);
+        R c[4];
+        c[0] = C2.x + C2.y;
+        c[1] = C3.x + C3.y;
+        if (q <= tiny * tiny) {  // |e| <= 4 size; c_2 may have underflowed
+            e = R(0);
+            return true;
+        }
+        if (sizeof(R) == 4 && q <= few * few) {
+            e = -c[1] * rcp_fast(c[0] + c[1]);
+            return true;
+        }
+        Two<R> C4 = two(R(0)), C5 = two(R(0));
+#pragma unroll
+        for (int k = 0; k < Q / 2; ++k) {
+            const Two<R> Ab = A[k] * b1[k], A2 = A[k] * A[k], b11 = b1[k] * b1[k], kA2 = kp[k] * A2;
+            const Two<R> n2 = fma2(kp[k], fma2(two(R(2)), Ab, A2), (two(R(-1)) * e1[k]) * b1[k]);
+            const Two<R> b2 = n2 * L[k];
+            C4 = fma2(w[k], fma2(two(R(0.5)) * b2, n2, kA2 * b11), C4);
+            const Two<R> in = fma2(b2, fma2(two(R(2)), A[k], b1[k]), two(R(2)) * Ab * (b1[k] + A[k]));
+            const Two<R> s5 = fma2(kp[k] * b2, in, kA2 * (b11 * b1[k]));
+            C5 = fma2(w[k], fma2(two(R(-0.5)) * e1[k], b2 * b2, s5), C5);
+            if constexpr (DIM == 2) {
+                const Two<R> z = zt[k] * e1[k];
+                C4 = C4 + z;
+                C5 = fma2(two(R(-1)) * z, e1[k], C5);
+            }
+        }
+        c[2] = C4.x + C4.y;
+        c[3] = C5.x + C5.y;
+        e = expansion_root<R, 4>(c, sizeof(R) == 4 ? 0 : 1);
+        return true;
+    }
+};
+
 // Cells too rough for the truncated expansion: Newton on B(t) - B(-1) from its root; then the general search.
 template <class Sys, class R>
 __host__ __device__ __forceinline__ bool rough_root(const ParamsR<R> &P, const R *u, const R *delta, R &omega)
@@ -363,15 +553,10 @@ __device__ __noinline__ R rough_omega(const ParamsR<R> &P, const R *u, const R *
 template <class Sys, class R>
 __device__ __forceinline__ R omega_of(const ParamsR<R> &P, const R *u, const R *delta, bool &fallback)
 {
-    using X = Expansion<Sys, R>;
-    X x;
-    if (x.build(P, u, delta) && x.size <= X::most) {
-        // |e| <= 4 size: below a quarter of the last place omega is 2 (and c_2 may have underflowed)
-        const R e = x.size <= Eps<R>::value / R(16) ? R(0) : expansion_root<R, X::N>(x.c, X::STEPS);
-        if (R(1) + e < P.t_max) {
-            fallback = false;
-            return R(2) + e;
-        }
+    R e;
+    if (SmoothRoot<Sys, R>::find(P, u, delta, e) && R(1) + e < P.t_max) {
+        fallback = false;
+        return R(2) + e;
     }
     R uu[Sys::M], dd[Sys::Q * Sys::M];
 #pragma unroll

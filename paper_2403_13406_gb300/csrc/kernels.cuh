@@ -23,13 +23,14 @@ constexpr int kRedThreads = 256;
 
 // Resident blocks of kBlock threads per SM that the relaxation's registers are held to.  The entropic
 // relaxations' out-of-line root-find of rough cells would otherwise set the registers of the whole kernel
-// (FP32 shallow water: 176, one block per SM; its common path needs 64 to 80).
+// (FP32 2D shallow water: 176, one block per SM).  Measured, FP32: 2D shallow water, 24 lattices, 4 steps: 22.3 ms
+// at two blocks, 25.1 at three, 28.0 at four (the common path spills); 2D Burgers 4096^2, 4 steps: 8.8 ms at
+// four, 11.4 at five.
 template <class Sys, class R, int OM> constexpr int relax_min_blocks()
 {
     if (OM == OM_FIXED || Sys::LINEAR) return 1;
     if (sizeof(R) == 8) return Sys::M == 1 ? 2 : 1;
-    if (OM == OM_MIXED) return 2;
-    return Sys::M == 1 ? 4 : 3;
+    return Sys::M == 1 && OM != OM_MIXED ? 4 : 2;
 }
 
 template <class R> struct StageArgs {
