@@ -144,11 +144,18 @@ constexpr int kStep2dMaxRing = 64;
 constexpr int kStep2dBarBytes = 8 * kStep2dMaxRing;
 constexpr int kStep2dSmemBudget = 232448 / kStep2dBlocksPerSm - 2048;
 
+// The temporally blocked 2D kernel in its form for FP32 Euler: one item a consumer, plane rows of a
+// compile-time length (13 ring rows of 16 planes of it are 208 KB).  Euler 8192^2, 3 steps: 64.4 ms; with rows of
+// 224, 192 and 160 values and up to 8 to 12 rows ahead 82.7, 77.2 and 94.4 ms (a tick takes about as long however
+// short its rows are).
+constexpr int kStep2dOneStride = 256;
+
 // Launch plan of the temporally blocked 2D kernel (k_step2d) for one group of
 // stages: a block owns tx x ly output cells and keeps `ring` rows of a window
 // tx + 2 hl wide in shared memory (see step2d.cuh).
 struct Plan2d {
     int tx, ly, hl, wx, ring, prefetch, nstrips, nsegs;
+    bool one;     // one item a consumer, plane rows kStep2dOneStride long
     int items;    // (stage, column) items of a tick: sum over the stages of tx + 2 (H - m_j)
     size_t smem;  // dynamic shared memory bytes
 };

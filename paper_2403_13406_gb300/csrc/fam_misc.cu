@@ -310,7 +310,12 @@ bool plan_step2d(int64_t nx, int64_t ny, int planes, int elem, int sms, const St
     if (pl.ring > kStep2dMaxRing) return false;
     pl.hl = (H + V4 - 1) / V4 * V4;
     const int64_t budget = kStep2dSmemBudget - kStep2dBarBytes;
-    const int wx_max = (int)(budget / ((int64_t)pl.ring * planes * elem)) / V4 * V4;
+    int wx_max = (int)(budget / ((int64_t)pl.ring * planes * elem)) / V4 * V4;
+    // 16 FP32 planes: the form with one item a consumer, where its longer plane rows fit (a narrower window,
+    // 248 instead of 284 columns for two stages) and a tick's items do not exceed the consumers
+    pl.one = planes == 16 && elem == 4 && (int64_t)pl.ring * 16 * kStep2dOneStride * 4 <= budget &&
+             sl.n * kStep2dOneStride <= kStep2dThreads - 32;
+    if (pl.one) wx_max = std::min(wx_max, kStep2dOneStride);
     const int tx_max = wx_max - 2 * pl.hl;
     // a tick's items (about n tx) must fit the slots of the smallest block
     const int tx_cap = (int)std::min<int64_t>(tx_max, (kStep2dMaxItems - items_margin) / sl.n / V4 * V4);

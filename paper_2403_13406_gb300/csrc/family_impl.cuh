@@ -262,17 +262,32 @@ cudaError_t step2d_one(const Step2dLaunch &L)
     const int nslots = (pl.items + cmax - 1) / cmax;
     if (nslots < 1 || nslots > kStep2dSlots) return cudaErrorInvalidValue;
     const int threads = 32 + ((pl.items + nslots - 1) / nslots + 31) / 32 * 32;
+    Step2dArgs<R> a{(const R *)L.fin, (R *)L.fout, L.nx, L.ny, L.ncell, pl.tx, pl.ly, pl.hl, pl.wx, pl.ring,
+                    pl.prefetch, pl.nstrips, L.cnt};
+    const unsigned grid = (unsigned)((int64_t)pl.nstrips * pl.nsegs);
     static std::atomic<int> attr[kMaxDevices];
     const int d = device_slot();
+    if constexpr (Sys::M == 4 && sizeof(R) == 4 && OM == OM_FIXED) {
+        if (pl.one && nslots == 1 && !L.P.shifted) {
+            static std::atomic<int> attr_one[kMaxDevices];
+            if (!attr_one[d].load()) {
+                cudaError_t e = cudaFuncSetAttribute(k_step2d<Sys, R, OM, true>,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, kStep2dSmemBudget);
+                if (e != cudaSuccess) return e;
+                attr_one[d].store(1);
+            }
+            const size_t smem = (size_t)kStep2dBarBytes + (size_t)pl.ring * 16 * kStep2dOneStride * sizeof(R);
+            if (pl.wx > kStep2dOneStride || smem > (size_t)kStep2dSmemBudget) return cudaErrorInvalidValue;
+            k_step2d<Sys, R, OM, true><<<grid, threads, smem, L.stream>>>(a, L.sl, params_as<R>(L.P));
+            return cudaGetLastError();
+        }
+    }
     if (!attr[d].load()) {
         cudaError_t e = cudaFuncSetAttribute(k_step2d<Sys, R, OM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kStep2dSmemBudget);
         if (e != cudaSuccess) return e;
         attr[d].store(1);
     }
-    Step2dArgs<R> a{(const R *)L.fin, (R *)L.fout, L.nx, L.ny, L.ncell, pl.tx, pl.ly, pl.hl, pl.wx, pl.ring,
-                    pl.prefetch, pl.nstrips, L.cnt};
-    const unsigned grid = (unsigned)((int64_t)pl.nstrips * pl.nsegs);
     k_step2d<Sys, R, OM><<<grid, threads, pl.smem, L.stream>>>(a, L.sl, params_as<R>(L.P));
     return cudaGetLastError();
 }

@@ -221,6 +221,48 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
     }
 }
 
+// The FP32 Euler relaxation with a fixed omega in packed pairs of components (0, 1) and (2, 3): the
+// operations and roundings of moments_target, deviations and the update, half the instructions
+// (plain storage; 1021 x 765, scheme III, 10 steps: 4.04 -> 3.87 ms).  The contractions are explicit, so that every kernel computes the same values.
+__device__ __forceinline__ void relax_euler_pairs(const ParamsR<float> &P, float *f, float w)
+{
+    const Two<float> minus = two(-1.0f), half = two(P.inv2V);
+    Two<float> F[4][2], u[2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) F[k][h] = two(f[k * 4 + 2 * h], f[k * 4 + 2 * h + 1]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) u[h] = ((F[0][h] + F[1][h]) + F[2][h]) + F[3][h];
+    const float mx = u[0].y, my = u[1].x, E = u[1].y;
+    const float rr = qdiv(1.0f, u[0].x);
+    const float vx = mx * rr, vy = my * rr;
+    const float p = P.gamma_m1 * fmaf(-0.5f, fmaf(my, vy, mx * vx), E);
+    const float H = E + p;
+    const Two<float> ph[2][2] = {{two(mx, fmaf(mx, vx, p)), two(my * vx, vx * H)},
+                                 {two(my, mx * vy), two(fmaf(my, vy, p), vy * H)}};
+    const Two<float> w2 = two(w);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const Two<float> base = u[h] * two(0.25f);
+        const Two<float> dx = ph[0][h] * half, dy = ph[1][h] * half;
+        const Two<float> d0 = fma2(minus, F[0][h], base + dx);
+        const Two<float> d1 = fma2(minus, F[1][h], base + dy);
+        const Two<float> d2 = fma2(minus, F[2][h], fma2(minus, dx, base));
+        const Two<float> s = (d0 + d1) + d2;
+        const Two<float> r0 = fma2(w2, d0, F[0][h]), r1 = fma2(w2, d1, F[1][h]), r2 = fma2(w2, d2, F[2][h]);
+        const Two<float> r3 = fma2(two(-w), s, F[3][h]);
+        f[2 * h] = r0.x;
+        f[2 * h + 1] = r0.y;
+        f[4 + 2 * h] = r1.x;
+        f[4 + 2 * h + 1] = r1.y;
+        f[8 + 2 * h] = r2.x;
+        f[8 + 2 * h + 1] = r2.y;
+        f[12 + 2 * h] = r3.x;
+        f[12 + 2 * h + 1] = r3.y;
+    }
+}
+
 // One relaxation of one cell (eq. relaxationDiscretizationOmega), in place.
 // rec: this relaxation's record (diagnostics, see Params::rec) or null; the
 // record only stores values the relaxation computes anyway.
@@ -228,6 +270,13 @@ template <class Sys, class R, int OM>
 __device__ __forceinline__ void relax_cell(const ParamsR<R> &P, R *f, int kind, bool &fallback, R *rec)
 {
     constexpr int Q = Sys::Q, M = Sys::M;
+    if constexpr (M == 4 && sizeof(R) == 4) {
+        if (!P.shifted) {
+            fallback = false;
+            relax_euler_pairs(P, f, kind == KIND_PROJECT ? 1.0f : P.omega);
+            return;
+        }
+    }
     const int64_t fs = (int64_t)P.rec_stages * P.rec_cells;  // distance between the fields of a record
     R u[M], feq[Q * M];
     moments_target<Sys, R>(P, f, u, feq);
