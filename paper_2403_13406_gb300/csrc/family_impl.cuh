@@ -83,9 +83,14 @@ cudaError_t stage_family(bool fp64, int om, const StageLaunch &L)
 // Tile of the temporally blocked 1D kernel: enough tiles to give every SM
 // `bps` resident blocks in a single wave, with the window of a block taking
 // at most its share of the SM's shared memory.
+// fp64_bound (FP64 storage and the mixed mode): a step takes what the FP64 pipe of the busiest SM takes, about
+// (tile + halo) cells per block and stage, so up to kBlock cells an SM one tile goes to each SM, however
+// short (a second block's halo costs more than it overlaps); at least 8 cells.  With 128 cells a tile against that:
+// 1D Burgers N = 256, FP64, 8 steps 1.76 -> 1.45 ms; 1D shallow water N = 30001, mixed, 6 steps 2.30 -> 1.75 ms.  The FP32 relaxations keep
+// tiles of 128 cells or more, whose halo they would feel.
 constexpr int kSmemPerSm = 220 * 1024;
 
-inline int fused_tile(int64_t n, int halo, int bytes_per_cell, int bps)
+inline int fused_tile(int64_t n, int halo, int bytes_per_cell, int bps, bool fp64_bound)
 {
     static std::atomic<int> sm_count[kMaxDevices];
     const int d = device_slot();
@@ -100,7 +105,9 @@ inline int fused_tile(int64_t n, int halo, int bytes_per_cell, int bps)
     int64_t t = (n + (int64_t)bps * sms - 1) / ((int64_t)bps * sms);
     t = ((t + 31) / 32) * 32;
     if (t < 128) t = 128;
+    if (fp64_bound && n <= (int64_t)kBlock * sms) t = std::max<int64_t>(8, ((n + sms - 1) / sms + 7) / 8 * 8);
     const int64_t tmax = (kSmemPerSm / bps) / bytes_per_cell - 2 * halo;
+    if (tmax < 32) return 0;  // the window does not fit
     if (t > tmax) t = tmax;
     return (int)t;
 }
@@ -123,8 +130,8 @@ cudaError_t fused_one_rec(const FusedLaunch &L)
         bps = occ < 1 ? 1 : (occ > 4 ? 4 : occ);
         bps_cache[d].store(bps);
     }
-    const int tile = fused_tile(L.n, L.sl.halo, NP * (int)sizeof(R), bps);
-    if (tile < 32) return cudaErrorInvalidValue;
+    const int tile = fused_tile(L.n, L.sl.halo, NP * (int)sizeof(R), bps, sizeof(R) == 8 || OM == OM_MIXED);
+    if (tile < 1) return cudaErrorInvalidValue;
     const size_t smem = (size_t)(tile + 2 * L.sl.halo) * NP * sizeof(R);
     FusedArgs<R> a{(const R *)L.fin, (R *)L.fout, L.n, tile, L.cnt,
                    (R *)L.rec, L.rec_stride_bytes / (int64_t)sizeof(R), L.nrec};
@@ -149,10 +156,13 @@ cudaError_t fused_family(bool fp64, int om, const FusedLaunch &L)
 template <class Sys, int DIM, class R>
 cudaError_t adjoint_prec(int om, const AdjointLaunch &L)
 {
-    dim3 grid((unsigned)((L.nx + kBlock - 1) / kBlock), (unsigned)L.ny);
+    // FP64: bound by the FP64 pipe, so blocks of 64 cells, which spread a short row over all SMs
+    // (with the tiles above, the gradient of 1D shallow water N = 16384, 4 steps: 15.1 -> 7.2 ms)
+    const unsigned block = sizeof(R) == 8 ? 64 : kBlock;
+    dim3 grid((unsigned)((L.nx + block - 1) / block), (unsigned)L.ny);
     const ParamsR<R> P = params_as<R>(L.P);
     return with_variant<Sys, R>(om, [&]<int OM>() {
-        k_adjoint_stage<Sys, DIM, R, OM><<<grid, kBlock, 0, L.stream>>>((const R *)L.fin, (const R *)L.gout,
+        k_adjoint_stage<Sys, DIM, R, OM><<<grid, block, 0, L.stream>>>((const R *)L.fin, (const R *)L.gout,
                                                                         (R *)L.gin, L.nx, L.ny, L.sh, L.kind, P);
         return cudaGetLastError();
     });
