@@ -48,10 +48,6 @@ SW_UREF = (1.0, 0.0)  # reference state of the shifted FP32 storage: the backgro
 BURGERS_N, BURGERS_V, BURGERS_STEPS = 4096, 3.0, 2000
 RIEMANN_N, RIEMANN_STEPS = 4096, 500
 BATCH_V, BATCH_STEPS, BATCH_K = 8.0, 500, 50
-# FP32 ALU roofline of the 1D entropic kernel (an explanation next to the HBM model there):
-# 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz, 415 FP32 flops per cell-stage (ncu count)
-FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-SW_FLOPS_PER_CELL_STAGE = 415.0
 
 
 def parse():
@@ -378,11 +374,8 @@ def sw1d_leg(torch, eslbm, inputs, stream, dev):
     planes = int(sim.sizes.planes)
     sim.close()
     s = ms * 1e-3
-    flops = SW_FLOPS_PER_CELL_STAGE * N * 18 * n_steps / s / 1e12
     roof = hbm_roofline(18 * 2 * planes * 4, N * n_steps, s, "k_step1d<ShallowWater<1>, float, entropic>",
-                        n_steps, {"alu_view": {"achieved_tflops": flops, "peak_tflops": FP32_PEAK_TFLOPS,
-                                               "frac": flops / FP32_PEAK_TFLOPS,
-                                               "flops_per_cell_stage": SW_FLOPS_PER_CELL_STAGE}},
+                        n_steps,
                         traffic=None)  # the capture predates the kernel's current D1Q2 deviations
     return {"sw1d": {"workload": "sw1d_d1q2_entropic_n%d_t%g" % (N, SW_T), "N": N, "V": SW_V, "g": G,
                      "t_final": n_steps * 24.0 / N / SW_V, "composite_steps": n_steps, "ms": ms,
