@@ -90,6 +90,15 @@ template <class R> struct Eps;
 template <> struct Eps<float> { static constexpr float value = 1.1920929e-7f; };
 template <> struct Eps<double> { static constexpr double value = 2.220446049250313e-16; };
 
+// Positive and far enough from the ends of the range that rcp_fast neither takes it for zero nor flushes its
+// reciprocal.  c_2 scales with the square of the fields (h V^2 size^2): thin films, h of 1e-21 and below in FP32, reach the
+// subnormal numbers while the deviation is ordinary, and -c_3 / (c_2 + c_3) would come out as -infinity.
+// Such cells go to the general search.
+template <class R> __host__ __device__ __forceinline__ bool ordinary(R x)
+{
+    return x >= R(sizeof(R) == 4 ? 0x1p-124 : 0x1p-1020) && x <= R(sizeof(R) == 4 ? 0x1p124 : 0x1p1020);
+}
+
 // Root e of H(e) with c[n] the coefficient of t^(n + 2), N of them: the quadratic model of H about 0 (exact to
 // e^5 relative to c_2), then in FP64 `steps` Newton steps on all of H.
 template <class R, int N> __host__ __device__ __forceinline__ R expansion_root(const R *c, int steps)
@@ -396,13 +405,15 @@ template <int DIM, class R> struct SmoothRoot<Scalar<DIM, true>, R> {
         const R s0 = S0.x + S0.y, s1 = S1.x + S1.y;
         if (sizeof(R) == 4 && q <= few * few) {
             const R c3 = s1 * R(2.0 / 3.0);  // over c_2 = s0 / 2
-            e = q <= tiny * tiny ? R(0) : -c3 * rcp_fast(s0 + c3);
-            return true;
+            const bool rest = q <= tiny * tiny;
+            e = rest ? R(0) : -c3 * rcp_fast(s0 + c3);
+            return rest || ordinary(s0);
         }
         if (q <= tiny * tiny) {
             e = R(0);
             return true;
         }
+        if (!ordinary(s0)) return false;
         constexpr double cat[8] = {1.0 / 2, 1.0 / 3, 2.0 / 4, 5.0 / 5, 14.0 / 6, 42.0 / 7, 132.0 / 8, 429.0 / 9};
         R c[N];
         c[0] = R(cat[0]) * s0;
@@ -434,7 +445,7 @@ template <int DIM, class R> struct SmoothRoot<ShallowWater<DIM>, R> {
         const R gh = P.g * u[0], gh2 = R(0.5) * gh;
         const R hV = u[0] * P.inv2V;
         const R nu = R(2) * P.V / R(Q);
-        bool ok = u[0] > R(0);
+        bool ok = ordinary(u[0]);
         Two<R> C2 = two(R(0)), C3 = two(R(0)), sq = two(R(0));
         Two<R> kp[Q / 2], e1[Q / 2], A[Q / 2], b1[Q / 2], w[Q / 2], L[Q / 2], zt[Q / 2];
 #pragma unroll
@@ -481,6 +492,7 @@ template <int DIM, class R> struct SmoothRoot<ShallowWater<DIM>, R> {
             e = R(0);
             return true;
         }
+        if (!ordinary(c[0])) return false;
         if (sizeof(R) == 4 && q <= few * few) {
             e = -c[1] * rcp_fast(c[0] + c[1]);
             return true;
@@ -522,7 +534,7 @@ __host__ __device__ __forceinline__ bool rough_root(const ParamsR<R> &P, const R
     R dt = R(1), dB = R(1);
     for (int it = 0; it < 8; ++it) {
         R B;
-        if (!X.eval(t, B, dB) || !(dB > R(0))) return false;
+        if (!X.eval(t, B, dB) || !ordinary(dB)) return false;
         dt = (B - E0) * rcp_fast(dB);
         t -= dt;
         if (!(t > R(0.1) && t < R(2.5))) return false;
@@ -554,7 +566,8 @@ template <class Sys, class R>
 __device__ __forceinline__ R omega_of(const ParamsR<R> &P, const R *u, const R *delta, bool &fallback)
 {
     R e;
-    if (SmoothRoot<Sys, R>::find(P, u, delta, e) && R(1) + e < P.t_max) {
+    // (a smooth cell's |e| is a few times its size, at most 0.2)
+    if (SmoothRoot<Sys, R>::find(P, u, delta, e) && fabs(e) < R(0.5) && R(1) + e < P.t_max) {
         fallback = false;
         return R(2) + e;
     }
