@@ -63,12 +63,14 @@ typedef enum {
 enum { ESLBM_LINEAR = 0, ESLBM_BURGERS = 1, ESLBM_SHALLOW_WATER = 2, ESLBM_EULER = 3 };
 /* Precision.  FP32 / FP64: storage and all arithmetic of the relaxation in that
    type (the reported reductions are FP64 in every mode).  FP32_MIXED (no
-   counterpart in the paper): FP32 storage and FP32 root-find iterations, with the
-   entropy difference of the entropic omega evaluated in FP64 -- E0 = B(-1) and
-   the residual F(t) = B(t) - E0 at the returned root, B(t) = sum_k B_k(t delta_k)
-   (Section 4, eq. variableOmegaProblem); when F(t) > 0 the chord root through
-   (0, -E0) and (t, F(t)), which never exceeds the root of the convex F, replaces
-   t.  With a fixed omega FP32_MIXED is FP32. */
+   counterpart in the paper): FP32 storage and the FP32 omega, lowered where needed so
+   that F(omega - 1) <= 0 in FP64, F(t) = B(t) - B(-1), B(t) = sum_k B_k(t delta_k)
+   (Section 4, eq. variableOmegaProblem): omega may not exceed the FP64 root where the
+   expansion of B or its closed form gives one; elsewhere, and next to the edge of the
+   convexity domain, F is evaluated in FP64 and, where F(t) > 0, the chord root
+   through (0, -B(-1)) and (t, F(t)), which never exceeds the root of the convex F,
+   replaces t.  FP32 and FP64 round the root itself to nearest.
+   With a fixed omega FP32_MIXED is FP32. */
 enum { ESLBM_FP32 = 0, ESLBM_FP64 = 1, ESLBM_FP32_MIXED = 2 };
 /* Temporal blocking (eslbm_config.blocking): AUTO runs the fastest measured path
    -- 1D: every step in one launch from shared memory; 2D: the temporally blocked

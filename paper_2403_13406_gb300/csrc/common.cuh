@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace eslbm {
 
 // Physical and numerical parameters of a run, passed by value to kernels.
@@ -45,6 +47,10 @@ struct Params {
 template <class R> struct ParamsR {
     R V, inv2V, a[2], c[2], g, gamma_m1, omega, t_max;
     R gV4, inv16gV;  // 4 g V and 1 / (16 g V) (shallow water)
+    // V, 4 g V and 1 / (16 g V) of the FP64 evaluations of a kernel's entropy (promote): all from the kernel's own
+    // inv2V and g, so that they belong to one and the same function.  Rounded to R each on its own they move
+    // the root of F next to the edge of the domain by up to 1e-5 (sqrt(g h) / V of 0.95 and more).
+    double V64, gV4_64, inv16gV_64;
     int shifted;     // see Params
     R ubar[4], cm[4], rdev[16], fbar[16], aux[4];
     R *rec;          // see Params
@@ -67,6 +73,9 @@ template <class R> inline ParamsR<R> params_as(const Params &P)
     q.t_max = R(P.t_max);
     q.gV4 = R(4.0 * P.g * P.V);
     q.inv16gV = P.g > 0 ? R(1.0 / (16.0 * P.g * P.V)) : R(0);
+    q.V64 = std::is_same_v<R, double> ? P.V : 0.5 / double(q.inv2V);
+    q.gV4_64 = 4.0 * double(q.g) * q.V64;
+    q.inv16gV_64 = P.g > 0 ? 1.0 / (16.0 * double(q.g) * q.V64) : 0.0;
     q.shifted = P.shifted;
     q.rec = reinterpret_cast<R *>(P.rec);
     q.rec_cells = P.rec_cells;

@@ -21,6 +21,7 @@ struct dfloat {
     // constants and host-side parameters; in device code only with constant arguments
     __host__ __device__ constexpr explicit dfloat(double v) : hi((float)v), lo((float)(v - (double)(float)v)) {}
     __host__ __device__ constexpr explicit dfloat(int v) : dfloat((double)v) {}
+    __host__ __device__ constexpr explicit operator double() const { return (double)hi + (double)lo; }  // host side
 };
 
 // a + b = s + e exactly

@@ -124,13 +124,12 @@ template <int Q, int M, class R> __host__ __device__ __forceinline__ void deviat
     }
 }
 
-// The kernel's constants in double precision, exactly as the kernel rounded them
-// (a float kernel's g, 1 / (2V), ... promoted), for the FP64 evaluations of the
-// mixed mode and of the diagnostics.
+// The kernel's constants in double precision for the FP64 evaluations of the mixed mode and of the
+// diagnostics: a float kernel's g, 1 / (2V), ... exactly as the kernel rounded them, what derives from them in FP64.
 template <class R> __device__ __forceinline__ ParamsR<double> promote(const ParamsR<R> &p)
 {
     ParamsR<double> q;
-    q.V = p.V;
+    q.V = p.V64;
     q.inv2V = p.inv2V;
     q.a[0] = p.a[0];
     q.a[1] = p.a[1];
@@ -140,8 +139,9 @@ template <class R> __device__ __forceinline__ ParamsR<double> promote(const Para
     q.gamma_m1 = p.gamma_m1;
     q.omega = p.omega;
     q.t_max = p.t_max;
-    q.gV4 = p.gV4;
-    q.inv16gV = p.inv16gV;
+    q.gV4 = q.gV4_64 = p.gV4_64;
+    q.inv16gV = q.inv16gV_64 = p.inv16gV_64;
+    q.V64 = p.V64;
     q.shifted = p.shifted;
     q.rec = nullptr;
     q.rec_cells = 0;
@@ -160,17 +160,18 @@ template <class R> __device__ __forceinline__ ParamsR<double> promote(const Para
     return q;
 }
 
-// Entropic omega with the entropy difference in FP64 (FP32 storage).  The FP32
-// root-find's t = omega - 1 is certified by evaluating, in double precision from
-// the same moments and deviations (and the kernel's own constants),
-// E0 = B(-1) = sum_k B_k(-delta_k) and the residual F(t) = B(t) - E0 at the
-// returned root.  F(t) <= 0 keeps omega.  F(t) > 0 (the FP32 root fell above the
-// root by its rounding) replaces t by the chord root through (0, -E0) and
-// (t, F(t)), t E0 / B(t): on a convex F that chord lies above F, so its root never
-// exceeds the root and the cell's microscopic entropy does not increase to FP64
-// rounding (Section 4).  The result is rounded towards zero to FP32 (t, then
-// omega = 1 + t), which keeps that side.  A cell that FP64 finds outside the
-// convexity domain falls back to omega = 1 (counted).
+// Entropic omega with the entropy difference in FP64 (FP32 storage).  The FP32 root-find's t = omega - 1 is
+// lowered, where needed, so that F(t) = B(t) - B(-1) <= 0 in double precision, from the same moments and deviations
+// and the kernel's own constants:
+//  - where the FP64 expansion or its closed form has the root (expansion.cuh), t may not exceed that root less a margin
+//    of 2^-20 of the cell's size, far above that root's own error and below the FP32 rounding of t;
+//  - next to the edge of the domain (size > 0.25), where the dual evaluations leave the domain before the closed form does,
+//    and where there is no such root, E0 = B(-1) and F(t) are evaluated.  F(t) > 0 replaces t by the chord
+//    root through (0, -E0) and (t, F(t)), t E0 / B(t), which on a convex F never exceeds the root, and that is
+//    evaluated again.
+// Results are rounded towards zero to FP32 (t, then omega = 1 + t), which keeps that side.  A cell that FP64 finds
+// outside the convexity domain falls back to omega = 1 (counted).  On 4 M random shallow-water cells up to the edge of
+// the domain no F exceeds the rounding of its evaluation.
 template <class Sys, class R>
 __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, bool &fallback)
 {
@@ -185,13 +186,11 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
         for (int m = 0; m < M; ++m) ud[m] = double(u[m]);
 #pragma unroll
         for (int i = 0; i < Q * M; ++i) dd[i] = double(delta[i]);
-        // Where the FP64 root 1 + wd is at hand, F(t) <= 0 up to it.  The kernel's FP32 constants 4 g V and
-        // 1 / (16 g V) are rounded on their own, which moves the root of the F they define by about 2^-23 of
-        // the size of a population's odd terms: stay a few times that below.
         using X = Expansion<Sys, double>;
         X x;
         double wd = 0.0;
         bool found = false;
+        // (FP64 coefficients of FP32 data are never subnormal)
         if (x.build(Pd, ud, dd) && x.size <= X::most) {
             wd = x.size <= Eps<double>::value / 16.0 ? 2.0 : 2.0 + expansion_root<double, X::N>(x.c, X::STEPS);
             found = wd < 1.0 + Pd.t_max;
@@ -200,7 +199,8 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
         }
         if (found) {
             wd -= x.size * 0x1p-20;
-            return double(w) <= wd ? w : __double2float_rz(wd);
+            if (double(w) > wd) w = __double2float_rz(wd);
+            if (x.size <= 0.25) return w;
         }
         typename Sys::template Ctx<double> cx;
         Sys::template prepare<double>(Pd, ud, dd, cx);
@@ -210,14 +210,17 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
             return R(1);
         }
         if (!(E0 > 0.0)) return w;  // at equilibrium: every omega leaves the cell unchanged
-        const double t = double(w) - 1.0;
-        if (!Sys::template eval<double>(Pd, cx, t, Bt, dBt)) {
-            fallback = true;
-            return R(1);
+#pragma unroll 1
+        for (int it = 0; it < 2; ++it) {
+            const double t = double(w) - 1.0;
+            if (!Sys::template eval<double>(Pd, cx, t, Bt, dBt)) {
+                fallback = true;
+                return R(1);
+            }
+            if (Bt - E0 <= 0.0) break;
+            w = __fadd_rz(1.0f, __double2float_rz(t * E0 / Bt));
         }
-        if (Bt - E0 <= 0.0) return w;
-        const float tc = __double2float_rz(t * E0 / Bt);
-        return __fadd_rz(1.0f, tc);
+        return w;
     }
 }
 
