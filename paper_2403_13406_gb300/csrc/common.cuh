@@ -46,6 +46,7 @@ struct Params {
 // derived constants the kernels need.
 template <class R> struct ParamsR {
     R V, inv2V, a[2], c[2], g, gamma_m1, omega, t_max;
+    R e_max;         // t_max - 1: bound of omega - 2
     R gV4, inv16gV;  // 4 g V and 1 / (16 g V) (shallow water)
     // V, 4 g V and 1 / (16 g V) of the FP64 evaluations of a kernel's entropy (promote): all from the kernel's own
     // inv2V and g, so that they belong to one and the same function.  Rounded to R each on its own they move
@@ -71,6 +72,7 @@ template <class R> inline ParamsR<R> params_as(const Params &P)
     q.gamma_m1 = R(P.gamma - 1.0);
     q.omega = R(P.omega);
     q.t_max = R(P.t_max);
+    q.e_max = R(P.t_max - 1.0);
     q.gV4 = R(4.0 * P.g * P.V);
     q.inv16gV = P.g > 0 ? R(1.0 / (16.0 * P.g * P.V)) : R(0);
     q.V64 = std::is_same_v<R, double> ? P.V : 0.5 / double(q.inv2V);

@@ -91,9 +91,7 @@ template <> struct Eps<float> { static constexpr float value = 1.1920929e-7f; };
 template <> struct Eps<double> { static constexpr double value = 2.220446049250313e-16; };
 
 // Positive and far enough from the ends of the range that rcp_fast neither takes it for zero nor flushes its
-// reciprocal.  c_2 scales with the square of the fields (h V^2 size^2): thin films, h of 1e-21 and below in FP32, reach the
-// subnormal numbers while the deviation is ordinary, and -c_3 / (c_2 + c_3) would come out as -infinity.
-// Such cells go to the general search.
+// reciprocal (its argument is subnormal or above 2^126 in FP32, 2^1022 in FP64).
 template <class R> __host__ __device__ __forceinline__ bool ordinary(R x)
 {
     return x >= R(sizeof(R) == 4 ? 0x1p-124 : 0x1p-1020) && x <= R(sizeof(R) == 4 ? 0x1p124 : 0x1p1020);
@@ -370,7 +368,9 @@ template <class R> __host__ __device__ __forceinline__ Two<R> rcp2(const Two<R> 
 // SmoothRoot<Sys, R>::find: the root e of a smooth cell from the expansion (the terms of Expansion, in pairs of
 // populations); false where the cell is too rough for it or outside the domain.  Its measure of roughness is
 // the sum of squares sq of the terms' ratios.  Very smooth cells (FP32, up to `few`: the terms of order
-// size^3 in omega are below its rounding) need c_2 and c_3 only: e = -c_3 / (c_2 + c_3).  Worst error of omega on the
+// size^3 in omega are below its rounding) need c_2 and c_3 only: e = -c_3 / (c_2 + c_3).  c_2 scales with the square of
+// the fields (h V^2 size^2 for shallow water): in thin films, h of 1e-21 and below in FP32, it is subnormal while the
+// deviation is ordinary, rcp_fast takes it for zero and e is infinite or NaN, which omega_of refuses.  Worst error of omega on the
 // random cells above: FP32 scalar 4e-8 up to `few` and up to `most`, shallow water 5e-8 up to `few`, 1e-6 up to
 // `most` (next to the domain's edge; what Newton on the closed form gives there too), FP64 6e-17.
 template <class Sys, class R> struct SmoothRoot;
@@ -400,20 +400,19 @@ template <int DIM, class R> struct SmoothRoot<Scalar<DIM, true>, R> {
             S1 = S1 + p[k];
         }
         const R q = sq.x + sq.y;
-        if (!(ok && q <= most * most)) return false;
-        constexpr R tiny = Eps<R>::value / R(16);
         const R s0 = S0.x + S0.y, s1 = S1.x + S1.y;
+        // (2 c_2 from the top of the range: rcp_fast would flush its reciprocal)
+        if (!(ok && q <= most * most && s0 <= R(sizeof(R) == 4 ? 0x1p124 : 0x1p1020))) return false;
+        constexpr R tiny = Eps<R>::value / R(16);
         if (sizeof(R) == 4 && q <= few * few) {
             const R c3 = s1 * R(2.0 / 3.0);  // over c_2 = s0 / 2
-            const bool rest = q <= tiny * tiny;
-            e = rest ? R(0) : -c3 * rcp_fast(s0 + c3);
-            return rest || ordinary(s0);
+            e = q <= tiny * tiny ? R(0) : -c3 * rcp_fast(s0 + c3);
+            return true;
         }
         if (q <= tiny * tiny) {
             e = R(0);
             return true;
         }
-        if (!ordinary(s0)) return false;
         constexpr double cat[8] = {1.0 / 2, 1.0 / 3, 2.0 / 4, 5.0 / 5, 14.0 / 6, 42.0 / 7, 132.0 / 8, 429.0 / 9};
         R c[N];
         c[0] = R(cat[0]) * s0;
@@ -445,7 +444,7 @@ template <int DIM, class R> struct SmoothRoot<ShallowWater<DIM>, R> {
         const R gh = P.g * u[0], gh2 = R(0.5) * gh;
         const R hV = u[0] * P.inv2V;
         const R nu = R(2) * P.V / R(Q);
-        bool ok = ordinary(u[0]);
+        bool ok = u[0] > R(0);
         Two<R> C2 = two(R(0)), C3 = two(R(0)), sq = two(R(0));
         Two<R> kp[Q / 2], e1[Q / 2], A[Q / 2], b1[Q / 2], w[Q / 2], L[Q / 2], zt[Q / 2];
 #pragma unroll
@@ -492,7 +491,6 @@ template <int DIM, class R> struct SmoothRoot<ShallowWater<DIM>, R> {
             e = R(0);
             return true;
         }
-        if (!ordinary(c[0])) return false;
         if (sizeof(R) == 4 && q <= few * few) {
             e = -c[1] * rcp_fast(c[0] + c[1]);
             return true;
@@ -566,8 +564,8 @@ template <class Sys, class R>
 __device__ __forceinline__ R omega_of(const ParamsR<R> &P, const R *u, const R *delta, bool &fallback)
 {
     R e;
-    // (a smooth cell's |e| is a few times its size, at most 0.2)
-    if (SmoothRoot<Sys, R>::find(P, u, delta, e) && fabs(e) < R(0.5) && R(1) + e < P.t_max) {
+    // (a smooth cell's |e| is a few times its size, at most 0.2; the lower bound refuses -infinity)
+    if (SmoothRoot<Sys, R>::find(P, u, delta, e) && e > R(-0.5) && e < P.e_max) {
         fallback = false;
         return R(2) + e;
     }

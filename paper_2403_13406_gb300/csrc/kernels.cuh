@@ -139,6 +139,7 @@ template <class R> __device__ __forceinline__ ParamsR<double> promote(const Para
     q.gamma_m1 = p.gamma_m1;
     q.omega = p.omega;
     q.t_max = p.t_max;
+    q.e_max = p.e_max;
     q.gV4 = q.gV4_64 = p.gV4_64;
     q.inv16gV = q.inv16gV_64 = p.inv16gV_64;
     q.V64 = p.V64;
