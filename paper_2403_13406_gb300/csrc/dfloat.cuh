@@ -79,9 +79,10 @@ template <> __host__ __device__ __forceinline__ dfloat sub_rn<dfloat>(dfloat a, 
 #endif
 }
 
-// v as a pair, in integer arithmetic; false (v left to FP64) unless v is zero or between 2^-40 and 2^40, where
-// no product of three such numbers and no residual of one leaves FP32's range
-__device__ __forceinline__ bool to_pair(double v, dfloat &p)
+// v as a pair, in integer arithmetic; false (v left to FP64) unless v is zero or between 2^-LOW and 2^40: with LOW = 40
+// no product of three such numbers and no residual of one leaves FP32's range.  Deviations (LOW = 70) may be smaller:
+// what their products lose is below the smallest FP32 number.
+template <unsigned LOW = 40> __device__ __forceinline__ bool to_pair(double v, dfloat &p)
 {
     const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
     const uint32_t mag = h & 0x7fffffffu, sign = h & 0x80000000u;
@@ -90,7 +91,7 @@ __device__ __forceinline__ bool to_pair(double v, dfloat &p)
     const bool zero = (mag | l) == 0u;
     p = quick_sum(top, __fmul_rn((float)(l & 0x1fffffffu), unit));
     if (zero) p = dfloat(0.0f, 0.0f);
-    return zero || (mag >= ((1023u - 40u) << 20) && mag < ((1023u + 40u) << 20));
+    return zero || (mag >= ((1023u - LOW) << 20) && mag < ((1023u + 40u) << 20));
 }
 
 // out of line: inlined, its FP64 operations are issued ahead of the branch for every cell

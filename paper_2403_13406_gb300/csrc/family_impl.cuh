@@ -332,7 +332,16 @@ cudaError_t init_family(bool fp64, const double *u0, void *f, int64_t ncell, con
 {
     const unsigned grid = (unsigned)((ncell + kBlock - 1) / kBlock);
     const ParamsR<double> Pd = params_as<double>(P);
-    const ParamsR<dfloat> Pp = params_as<dfloat>(P);
+    ParamsR<dfloat> Pp = params_as<dfloat>(P);
+    if (P.shifted) {
+        // the reference's own terms with the parameters as given (P holds those of the storage precision's kernels)
+        double ub[4], feq[16];
+        for (int m = 0; m < 4; ++m) ub[m] = P.ubar[m];
+        Sys::template equilibrium<double>(Pd, ub, feq);
+        for (int i = 0; i < Sys::Q * Sys::M; ++i) Pp.rdev[i] = dfloat(feq[i] - P.fbar[i]);
+        if (Sys::M == 4)  // the reference pressure
+            Pp.aux[2] = dfloat(Pd.gamma_m1 * (ub[3] - 0.5 * (ub[1] * P.aux[0] + ub[2] * P.aux[1])));
+    }
     if (fp64) k_init_eq<Sys, double><<<grid, kBlock, 0, st>>>(u0, (double *)f, ncell, Pd, Pp, cnt);
     else k_init_eq<Sys, float><<<grid, kBlock, 0, st>>>(u0, (float *)f, ncell, Pd, Pp, cnt);
     return cudaGetLastError();

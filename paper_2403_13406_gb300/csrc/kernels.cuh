@@ -933,9 +933,39 @@ __device__ __noinline__ void init_cell_general(const ParamsR<double> &P, const d
     init_cell<Sys, R>(P, u, f, bad);
 }
 
-// FP32 lattices: the equilibrium in pairs of FP32 numbers (dfloat.cuh) rounded to FP32 at the end, where the
-// fields are of ordinary size and an FP32 test finds them inside the domain by a margin far above its
-// rounding; other cells in FP64.
+// The same for FP32 lattices in pairs of FP32 numbers (dfloat.cuh), rounded to FP32 at the end; false, and the cell
+// left to FP64, unless the fields are of ordinary size and an FP32 test finds them inside the domain by a margin far
+// above its rounding.  The shifted storage takes the deviation form: u - ubar is exact, and what the
+// pairs round is relative to the deviation, where f^eq - fbar from two pairs would keep 45 bits of f^eq only.
+template <class Sys>
+__device__ __forceinline__ bool init_pairs(const ParamsR<double> &P, const ParamsR<dfloat> &Pp, const double *u,
+                                           float *f)
+{
+    constexpr int M = Sys::M, NP = Sys::Q * M;
+    dfloat up[M], du[M], feq[NP];
+    float uf[M];
+    bool ok = true;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        ok &= to_pair(u[m], up[m]);
+        uf[m] = up[m].hi;
+    }
+    if (!ok || !Sys::well_inside(Pp, uf)) return false;
+    if (!P.shifted) {
+        Sys::template equilibrium<dfloat>(Pp, up, feq);
+#pragma unroll
+        for (int j = 0; j < NP; ++j) f[j] = feq[j].hi;
+        return true;
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m) ok &= to_pair<70>(u[m] - P.ubar[m], du[m]);
+    if (!ok) return false;
+    Sys::template equilibrium_dev<dfloat>(Pp, du, up, feq);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) f[j] = (feq[j] + Pp.rdev[j]).hi;
+    return true;
+}
+
 template <class Sys, class R>
 __global__ void __launch_bounds__(kBlock) k_init_eq(const double *__restrict__ u0, R *__restrict__ f,
                                                     int64_t ncell, const __grid_constant__ ParamsR<double> P,
@@ -953,20 +983,7 @@ __global__ void __launch_bounds__(kBlock) k_init_eq(const double *__restrict__ u
         }
         R out[Q * M];
         if constexpr (sizeof(R) == 4) {
-            dfloat up[M];
-            float uf[M];
-            bool ok = true;
-#pragma unroll
-            for (int m = 0; m < M; ++m) {
-                ok &= to_pair(u[m], up[m]);
-                uf[m] = up[m].hi;
-            }
-            if (ok && Sys::well_inside(Pp, uf)) {
-                dfloat feq[Q * M];
-                Sys::template equilibrium<dfloat>(Pp, up, feq);
-#pragma unroll
-                for (int j = 0; j < Q * M; ++j) out[j] = P.shifted ? (feq[j] - Pp.fbar[j]).hi : feq[j].hi;
-            } else {
+            if (!init_pairs<Sys>(P, Pp, u, out)) {
                 double uu[M];
 #pragma unroll
                 for (int m = 0; m < M; ++m) uu[m] = u[m];
