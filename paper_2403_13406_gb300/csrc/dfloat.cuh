@@ -3,7 +3,7 @@
 // The equilibrium of the initial fields and the moments read back are computed in 64 bits and then rounded
 // to, or summed from, FP32 values.  GB300's FP64 pipe does 2 operations a clock and SM, conversions
 // included, 1/64 of the FP32 rate, so these passes over HBM-resident fields were bound by it: 2D Euler 8192^2,
-// init 10.0 ms (now 1.34) and moments 6.0 ms against 0.95 ms of HBM each.  The pair operations below (error-free
+// init 10.0 ms (now 1.42) and moments 6.0 ms against 0.95 ms of HBM each.  The pair operations below (error-free
 // transformations of Dekker and Knuth with FMA) keep 45 bits or more at about ten FP32 instructions each.
 #pragma once
 
@@ -77,6 +77,55 @@ template <> __host__ __device__ __forceinline__ dfloat sub_rn<dfloat>(dfloat a, 
 #else
     return a;
 #endif
+}
+
+// Magnitudes: an expression in this type is the sum of the magnitudes of its terms, which bounds the terms that
+// cancel in the expression itself (and so, times 2^-44, the error of its value in pairs).
+struct fmag {
+    float v;
+    fmag() = default;
+    __host__ __device__ constexpr explicit fmag(float x) : v(x < 0.0f ? -x : x) {}
+    __host__ __device__ constexpr explicit fmag(double x) : fmag((float)x) {}
+    __host__ __device__ constexpr explicit fmag(int x) : fmag((float)x) {}
+    __device__ __forceinline__ explicit fmag(const dfloat &x) : v(fabsf(x.hi)) {}
+};
+__device__ __forceinline__ fmag operator+(const fmag &a, const fmag &b) { return fmag(a.v + b.v); }
+__device__ __forceinline__ fmag operator-(const fmag &a, const fmag &b) { return fmag(a.v + b.v); }
+__device__ __forceinline__ fmag operator*(const fmag &a, const fmag &b) { return fmag(a.v * b.v); }
+__device__ __forceinline__ fmag operator/(const fmag &a, const fmag &b) { return fmag(__fdividef(a.v, b.v)); }
+template <> __host__ __device__ __forceinline__ fmag add_rn<fmag>(fmag a, fmag b)
+{
+#ifdef __CUDA_ARCH__
+    return a + b;
+#else
+    return a;
+#endif
+}
+template <> __host__ __device__ __forceinline__ fmag sub_rn<fmag>(fmag a, fmag b)
+{
+#ifdef __CUDA_ARCH__
+    return a + b;
+#else
+    return a;
+#endif
+}
+// the constants that the equilibria read
+__device__ __forceinline__ ParamsR<fmag> magnitudes(const ParamsR<dfloat> &p)
+{
+    ParamsR<fmag> q;
+    q.V = fmag(p.V);
+    q.inv2V = fmag(p.inv2V);
+    for (int j = 0; j < 2; ++j) {
+        q.a[j] = fmag(p.a[j]);
+        q.c[j] = fmag(p.c[j]);
+    }
+    q.g = fmag(p.g);
+    q.gamma_m1 = fmag(p.gamma_m1);
+    for (int i = 0; i < 4; ++i) {
+        q.ubar[i] = fmag(p.ubar[i]);
+        q.aux[i] = fmag(p.aux[i]);
+    }
+    return q;
 }
 
 // v as a pair, in integer arithmetic; false (v left to FP64) unless v is zero or between 2^-LOW and 2^40: with LOW = 40

@@ -934,8 +934,9 @@ __device__ __noinline__ void init_cell_general(const ParamsR<double> &P, const d
 }
 
 // The same for FP32 lattices in pairs of FP32 numbers (dfloat.cuh), rounded to FP32 at the end; false, and the cell
-// left to FP64, unless the fields are of ordinary size and an FP32 test finds them inside the domain by a margin far
-// above its rounding.  The shifted storage takes the deviation form: u - ubar is exact, and what the
+// left to FP64, unless the fields are of ordinary size, an FP32 test finds them inside the domain by a margin far
+// above its rounding, and no population is what is left of terms 2^10 times as large (the pairs' 2^-44 of those
+// then stay 2^-10 below the rounding to FP32).  The shifted storage takes the deviation form: u - ubar is exact, and what the
 // pairs round is relative to the deviation, where f^eq - fbar from two pairs would keep 45 bits of f^eq only.
 template <class Sys>
 __device__ __forceinline__ bool init_pairs(const ParamsR<double> &P, const ParamsR<dfloat> &Pp, const double *u,
@@ -951,19 +952,36 @@ __device__ __forceinline__ bool init_pairs(const ParamsR<double> &P, const Param
         uf[m] = up[m].hi;
     }
     if (!ok || !Sys::well_inside(Pp, uf)) return false;
+    constexpr float few = 0x1p-10f;
     if (!P.shifted) {
+        // u_m / q +- phi / (2V): the larger of two opposite populations is the sum of the magnitudes of their terms
+        // (those of phi itself have one sign, but for the Euler pressure's, which well_inside holds to 1e-4)
         Sys::template equilibrium<dfloat>(Pp, up, feq);
 #pragma unroll
+        for (int j = 0; j < NP / 2; ++j) {
+            const float a = fabsf(feq[j].hi), b = fabsf(feq[j + NP / 2].hi);
+            ok &= fminf(a, b) >= few * fmaxf(a, b);
+        }
+#pragma unroll
         for (int j = 0; j < NP; ++j) f[j] = feq[j].hi;
-        return true;
+        return ok;
     }
+    fmag um[M], dm[M], mag[NP];
+    const ParamsR<fmag> Pm = magnitudes(Pp);
 #pragma unroll
-    for (int m = 0; m < M; ++m) ok &= to_pair<70>(u[m] - P.ubar[m], du[m]);
-    if (!ok) return false;
+    for (int m = 0; m < M; ++m) {
+        ok &= to_pair<70>(u[m] - P.ubar[m], du[m]);
+        um[m] = fmag(up[m]);
+        dm[m] = fmag(du[m]);
+    }
     Sys::template equilibrium_dev<dfloat>(Pp, du, up, feq);
+    Sys::template equilibrium_dev<fmag>(Pm, dm, um, mag);
 #pragma unroll
-    for (int j = 0; j < NP; ++j) f[j] = (feq[j] + Pp.rdev[j]).hi;
-    return true;
+    for (int j = 0; j < NP; ++j) {
+        f[j] = (feq[j] + Pp.rdev[j]).hi;
+        ok &= fabsf(f[j]) >= few * (mag[j] + fmag(Pp.rdev[j])).v;
+    }
+    return ok;
 }
 
 template <class Sys, class R>
