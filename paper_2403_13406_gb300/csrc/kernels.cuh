@@ -227,7 +227,8 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
 
 // The FP32 Euler relaxation with a fixed omega in packed pairs of components (0, 1) and (2, 3): the
 // operations and roundings of moments_target, deviations and the update, half the instructions
-// (plain storage; 1021 x 765, scheme III, 10 steps: 4.04 -> 3.87 ms).  The contractions are explicit, so that every kernel computes the same values.
+// (plain storage; 1021 x 765, scheme III, 10 steps: 4.04 -> 3.87 ms).  No sum of a product is left for the compiler to
+// contract or not, so every kernel computes the same values.
 __device__ __forceinline__ void relax_euler_pairs(const ParamsR<float> &P, float *f, float w)
 {
     const Two<float> minus = two(-1.0f), half = two(P.inv2V);
@@ -242,7 +243,7 @@ __device__ __forceinline__ void relax_euler_pairs(const ParamsR<float> &P, float
     const float rr = qdiv(1.0f, u[0].x);
     const float vx = mx * rr, vy = my * rr;
     const float p = P.gamma_m1 * fmaf(-0.5f, fmaf(my, vy, mx * vx), E);
-    const float H = E + p;
+    const float H = __fadd_rn(E, p);
     const Two<float> ph[2][2] = {{two(mx, fmaf(mx, vx, p)), two(my * vx, vx * H)},
                                  {two(my, mx * vy), two(fmaf(my, vy, p), vy * H)}};
     const Two<float> w2 = two(w);
