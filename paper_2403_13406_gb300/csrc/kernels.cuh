@@ -936,9 +936,10 @@ __device__ __noinline__ void init_cell_general(const ParamsR<double> &P, const d
 
 // The same for FP32 lattices in pairs of FP32 numbers (dfloat.cuh), rounded to FP32 at the end; false, and the cell
 // left to FP64, unless the fields are of ordinary size, an FP32 test finds them inside the domain by a margin far
-// above its rounding, and no population is what is left of terms 2^10 times as large (the pairs' 2^-44 of those
-// then stay 2^-10 below the rounding to FP32).  The shifted storage takes the deviation form: u - ubar is exact, and what the
-// pairs round is relative to the deviation, where f^eq - fbar from two pairs would keep 45 bits of f^eq only.
+// above its rounding, and no population is what is left of terms 2^12 times as large (the pairs' 2^-43 of those
+// then stay 2^-7 below the rounding to FP32; with 2^10 one warp in two has such a cell in a shifted vortex).  The shifted
+// storage takes the deviation form: u - ubar is exact, and what the pairs round is relative to the deviation, where
+// f^eq - fbar from two pairs would keep 45 bits of f^eq only.
 template <class Sys>
 __device__ __forceinline__ bool init_pairs(const ParamsR<double> &P, const ParamsR<dfloat> &Pp, const double *u,
                                            float *f)
@@ -953,7 +954,7 @@ __device__ __forceinline__ bool init_pairs(const ParamsR<double> &P, const Param
         uf[m] = up[m].hi;
     }
     if (!ok || !Sys::well_inside(Pp, uf)) return false;
-    constexpr float few = 0x1p-10f;
+    constexpr float few = 0x1p-12f;
     if (!P.shifted) {
         // u_m / q +- phi / (2V): the larger of two opposite populations is the sum of the magnitudes of their terms
         // (those of phi itself have one sign, but for the Euler pressure's, which well_inside holds to 1e-4)
