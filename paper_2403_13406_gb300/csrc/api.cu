@@ -311,7 +311,7 @@ bool step_groups2d(const eslbm_handle *h, int64_t pending, std::vector<Group2d> 
             G.sl.kind[j] = st[(size_t)(spans[i].first + j)].second;
             G.sl.halo += std::abs(G.sl.shift[j]);
         }
-        if (plan_step2d(h->cfg.nx, h->cfg.ny, (int)h->sz.planes, elem, sms, G.sl, G.plan)) {
+        if (plan_step2d(h->cfg.nx, h->cfg.ny, (int)h->sz.planes, elem, h->cfg.shifted != 0, sms, G.sl, G.plan)) {
             out.push_back(G);
         } else {
             if (G.sl.n == 1) return false;

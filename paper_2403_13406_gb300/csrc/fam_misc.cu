@@ -287,7 +287,7 @@ int device_sms()
     return sms;
 }
 
-bool plan_step2d(int64_t nx, int64_t ny, int planes, int elem, int sms, const StageList &sl, Plan2d &pl)
+bool plan_step2d(int64_t nx, int64_t ny, int planes, int elem, bool shifted, int sms, const StageList &sl, Plan2d &pl)
 {
     if (!stage_list_ok(sl) || sl.n > kStep2dMaxStages || planes < 1 || (elem != 4 && elem != 8)) return false;
     const int V4 = 16 / elem;
@@ -311,39 +311,49 @@ bool plan_step2d(int64_t nx, int64_t ny, int planes, int elem, int sms, const St
     pl.hl = (H + V4 - 1) / V4 * V4;
     const int64_t budget = kStep2dSmemBudget - kStep2dBarBytes;
     int wx_max = (int)(budget / ((int64_t)pl.ring * planes * elem)) / V4 * V4;
-    // 16 FP32 planes: the form with one item a consumer, where its longer plane rows fit (a narrower window,
-    // 248 instead of 284 columns for two stages) and a tick's items do not exceed the consumers
-    pl.one = planes == 16 && elem == 4 && (int64_t)pl.ring * 16 * kStep2dOneStride * 4 <= budget &&
+    // 16 FP32 planes in plain storage: the form with one item a consumer, where its longer plane rows fit (a narrower
+    // window, 248 instead of 276 columns for two stages) and a tick's items do not exceed the consumers
+    pl.one = planes == 16 && elem == 4 && !shifted && (int64_t)pl.ring * 16 * kStep2dOneStride * 4 <= budget &&
              sl.n * kStep2dOneStride <= kStep2dThreads - 32;
     if (pl.one) wx_max = std::min(wx_max, kStep2dOneStride);
-    const int tx_max = wx_max - 2 * pl.hl;
-    // a tick's items (about n tx) must fit the slots of the smallest block
-    const int tx_cap = (int)std::min<int64_t>(tx_max, (kStep2dMaxItems - items_margin) / sl.n / V4 * V4);
-    if (tx_cap < std::max(4 * V4, pl.hl)) return false;
-    // strips as wide as the window allows, evened out over the row
-    int64_t nstrips = (nx + tx_cap - 1) / tx_cap;
-    const int64_t even = (nx + nstrips - 1) / nstrips;
-    pl.tx = (int)((even + V4 - 1) / V4 * V4);
-    nstrips = (nx + pl.tx - 1) / pl.tx;
-    pl.nstrips = (int)nstrips;
-    pl.wx = pl.tx + 2 * pl.hl;
-    // rows per block: the time is (waves of kStep2dBlocksPerSm blocks per SM) x (ticks of a block)
-    static const int cand[] = {32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048, 3072, 4096, 8192};
+    // Strips as wide as the window allows, evened out over the row; rows per block: the time is (waves of
+    // kStep2dBlocksPerSm blocks per SM) x (ticks of a block).
     double best = 0.0;
     pl.ly = 0;
-    for (int ly : cand) {
-        const int lye = (int)std::min<int64_t>(ly, ny);
-        const int64_t nsegs = (ny + lye - 1) / lye;
-        const int64_t blocks = nstrips * nsegs;
-        const int64_t waves = (blocks + (int64_t)sms * kStep2dBlocksPerSm - 1) / ((int64_t)sms * kStep2dBlocksPerSm);
-        const double cost = (double)waves * (double)(lye + H + lag);
-        if (pl.ly == 0 || cost < best) {
-            best = cost;
-            pl.ly = lye;
-            pl.nsegs = (int)nsegs;
+    auto strips = [&](int tx_cap) {
+        int64_t nstrips = (nx + tx_cap - 1) / tx_cap;
+        const int64_t even = (nx + nstrips - 1) / nstrips;
+        const int tx = (int)((even + V4 - 1) / V4 * V4);
+        nstrips = (nx + tx - 1) / tx;
+        static const int cand[] = {32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048, 3072, 4096, 8192};
+        bool taken = false;
+        for (int ly : cand) {
+            const int lye = (int)std::min<int64_t>(ly, ny);
+            const int64_t nsegs = (ny + lye - 1) / lye;
+            const int64_t blocks = nstrips * nsegs;
+            const int64_t waves = (blocks + (int64_t)sms * kStep2dBlocksPerSm - 1) / ((int64_t)sms * kStep2dBlocksPerSm);
+            const double cost = (double)waves * (double)(lye + H + lag);
+            if (pl.ly == 0 || cost < best || (!taken && cost == best)) {
+                taken = true;
+                best = cost;
+                pl.ly = lye;
+                pl.nsegs = (int)nsegs;
+                pl.nstrips = (int)nstrips;
+                pl.tx = tx;
+            }
+            if (ly >= ny) break;
         }
-        if (ly >= ny) break;
-    }
+    };
+    // a tick's items (about n tx) must fit the slots of the smallest block
+    const int tx_items = (int)((kStep2dMaxItems - items_margin) / sl.n / V4 * V4);
+    const int tx_cap = std::min(wx_max - 2 * pl.hl, tx_items);
+    if (tx_cap < std::max(4 * V4, pl.hl)) return false;
+    strips(tx_cap);
+    // Shifted 16-plane states: strips of at most 248 columns where they cost no more ticks, which are then shorter.
+    // Euler, us a step, 276 columns / 248 / this rule: 512^2 692 / 596 / 596, 1024^2 722 / 890 / 723, 2048^2 2202 / 2092 / 2071,
+    // 4096^2 6545 / 8371 / 6543, 8192^2 21650 / 25446 / 21651.
+    if (planes == 16 && elem == 4 && shifted && tx_cap > kStep2dOneStride - 2 * pl.hl) strips(kStep2dOneStride - 2 * pl.hl);
+    pl.wx = pl.tx + 2 * pl.hl;
     if ((int64_t)pl.nstrips * pl.nsegs > 0x7fffffffLL) return false;
     pl.items = (int)((int64_t)sl.n * pl.tx + items_margin);
     pl.smem = (size_t)kStep2dBarBytes + (size_t)pl.ring * planes * pl.wx * elem;

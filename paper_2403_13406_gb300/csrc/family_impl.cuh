@@ -278,7 +278,7 @@ cudaError_t step2d_one(const Step2dLaunch &L)
     static std::atomic<int> attr[kMaxDevices];
     const int d = device_slot();
     if constexpr (Sys::M == 4 && sizeof(R) == 4 && OM == OM_FIXED) {
-        if (pl.one && nslots == 1 && !L.P.shifted) {
+        if (pl.one && nslots == 1) {
             static std::atomic<int> attr_one[kMaxDevices];
             if (!attr_one[d].load()) {
                 cudaError_t e = cudaFuncSetAttribute(k_step2d<Sys, R, OM, true>,
