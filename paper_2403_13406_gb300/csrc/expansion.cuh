@@ -92,9 +92,25 @@ template <> struct Eps<double> { static constexpr double value = 2.2204460492503
 
 // Positive and far enough from the ends of the range that rcp_fast neither takes it for zero nor flushes its
 // reciprocal (its argument is subnormal or above 2^126 in FP32, 2^1022 in FP64).
-template <class R> __host__ __device__ __forceinline__ bool ordinary(R x)
+// FP64: from the upper word, off the FP64 pipe.
+__host__ __device__ __forceinline__ bool ordinary(float x) { return x >= 0x1p-124f && x <= 0x1p124f; }
+__host__ __device__ __forceinline__ bool ordinary(double x)
 {
-    return x >= R(sizeof(R) == 4 ? 0x1p-124 : 0x1p-1020) && x <= R(sizeof(R) == 4 ? 0x1p124 : 0x1p1020);
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2hiint(x) - (3u << 20) < (2040u << 20);
+#else
+    return x >= 0x1p-1020 && x < 0x1p1020;
+#endif
+}
+// the upper bound alone, for x >= 0
+__host__ __device__ __forceinline__ bool below_top(float x) { return x <= 0x1p124f; }
+__host__ __device__ __forceinline__ bool below_top(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2hiint(x) < (2043u << 20);
+#else
+    return x < 0x1p1020;
+#endif
 }
 
 // Root e of H(e) with c[n] the coefficient of t^(n + 2), N of them: the quadratic model of H about 0 (exact to
@@ -402,7 +418,7 @@ template <int DIM, class R> struct SmoothRoot<Scalar<DIM, true>, R> {
         const R q = sq.x + sq.y;
         const R s0 = S0.x + S0.y, s1 = S1.x + S1.y;
         // (2 c_2 from the top of the range: rcp_fast would flush its reciprocal)
-        if (!(ok && q <= most * most && s0 <= R(sizeof(R) == 4 ? 0x1p124 : 0x1p1020))) return false;
+        if (!(ok && q <= most * most && below_top(s0))) return false;
         constexpr R tiny = Eps<R>::value / R(16);
         if (sizeof(R) == 4 && q <= few * few) {
             const R c3 = s1 * R(2.0 / 3.0);  // over c_2 = s0 / 2
