@@ -25,11 +25,11 @@ constexpr int kRedThreads = 256;
 // relaxations' out-of-line root-find of rough cells would otherwise set the registers of the whole kernel
 // (FP32 2D shallow water: 176, one block per SM).  Measured, FP32: 2D shallow water, 24 lattices, 4 steps: 22.3 ms
 // at two blocks, 25.1 at three, 28.0 at four (the common path spills); 2D Burgers 4096^2, 4 steps: 8.8 ms at
-// four, 11.4 at five.
+// four, 11.4 at five.  FP64, one step at one block / two: 2D Burgers 192^2 842 / 909 us, 384^2 1583 / 1610, 1021^2 6908 / 6908,
+// 2048^2 27.2 / 26.7 ms; 2D shallow water 192^2 3.06 / 3.11 ms, 2048^2 156 / 155.
 template <class Sys, class R, int OM> constexpr int relax_min_blocks()
 {
-    if (OM == OM_FIXED || Sys::LINEAR) return 1;
-    if (sizeof(R) == 8) return Sys::M == 1 ? 2 : 1;
+    if (OM == OM_FIXED || Sys::LINEAR || sizeof(R) == 8) return 1;
     return Sys::M == 1 && OM != OM_MIXED ? 4 : 2;
 }
 
