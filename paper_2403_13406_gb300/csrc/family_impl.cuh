@@ -83,14 +83,23 @@ cudaError_t stage_family(bool fp64, int om, const StageLaunch &L)
 // Tile of the temporally blocked 1D kernel: enough tiles to give every SM
 // `bps` resident blocks in a single wave, with the window of a block taking
 // at most its share of the SM's shared memory.
-// fp64_bound (FP64 storage and the mixed mode): a step takes what the FP64 pipe of the busiest SM takes, about
-// (tile + halo) cells per block and stage, so up to kBlock cells an SM one tile goes to each SM, however
+// one_tile (FP64 storage and the mixed mode; 0 otherwise): a step takes what the FP64 pipe of the busiest SM takes,
+// about (tile + halo) cells per block and stage, so up to that many cells an SM one tile goes to each SM, however
 // short (a second block's halo costs more than it overlaps); at least 8 cells.  With 128 cells a tile against that:
-// 1D Burgers N = 256, FP64, 8 steps 1.76 -> 1.45 ms; 1D shallow water N = 30001, mixed, 6 steps 2.30 -> 1.75 ms.  The FP32 relaxations keep
-// tiles of 128 cells or more, whose halo they would feel.
+// 1D Burgers N = 256, FP64, 8 steps 1.76 -> 1.45 ms; 1D shallow water N = 30001, mixed, 6 steps 2.30 -> 1.75 ms.
+// With more cells an SM two tiles of 128 fill the SMs as evenly and overlap.  FP64, 4 steps, one tile of 232 / 240 / 248 /
+// 256 cells an SM against two tiles: fixed omega, scheme I, linear 110 / 118 / 119 / 126 against 110 us, shallow water 234 /
+// 247 / 256 / 265 against 243; entropic, scheme I, Burgers 872 / 903 / 937 / 969 against 946, shallow water 1590 / 1648 / 1698 /
+// 1752 against 1688, mixed 3030 / 3150 / 3273 / 3395 against 3240; entropic, plain scheme, Burgers 44 / 44 / 44 / 57
+// against 52.  The FP32 relaxations keep tiles of 128 cells or more, whose halo they would feel.
+template <class R, int OM> constexpr int one_tile_cells()
+{
+    if (sizeof(R) == 4 && OM != OM_MIXED) return 0;
+    return OM == OM_FIXED ? 232 : 248;
+}
 constexpr int kSmemPerSm = 220 * 1024;
 
-inline int fused_tile(int64_t n, int halo, int bytes_per_cell, int bps, bool fp64_bound)
+inline int fused_tile(int64_t n, int halo, int bytes_per_cell, int bps, int one_tile)
 {
     static std::atomic<int> sm_count[kMaxDevices];
     const int d = device_slot();
@@ -105,7 +114,7 @@ inline int fused_tile(int64_t n, int halo, int bytes_per_cell, int bps, bool fp6
     int64_t t = (n + (int64_t)bps * sms - 1) / ((int64_t)bps * sms);
     t = ((t + 31) / 32) * 32;
     if (t < 128) t = 128;
-    if (fp64_bound && n <= (int64_t)kBlock * sms) t = std::max<int64_t>(8, ((n + sms - 1) / sms + 7) / 8 * 8);
+    if (n <= (int64_t)one_tile * sms) t = std::max<int64_t>(8, ((n + sms - 1) / sms + 7) / 8 * 8);
     const int64_t tmax = (kSmemPerSm / bps) / bytes_per_cell - 2 * halo;
     if (tmax < 32) return 0;  // the window does not fit
     if (t > tmax) t = tmax;
@@ -130,7 +139,7 @@ cudaError_t fused_one_rec(const FusedLaunch &L)
         bps = occ < 1 ? 1 : (occ > 4 ? 4 : occ);
         bps_cache[d].store(bps);
     }
-    const int tile = fused_tile(L.n, L.sl.halo, NP * (int)sizeof(R), bps, sizeof(R) == 8 || OM == OM_MIXED);
+    const int tile = fused_tile(L.n, L.sl.halo, NP * (int)sizeof(R), bps, one_tile_cells<R, OM>());
     if (tile < 1) return cudaErrorInvalidValue;
     const size_t smem = (size_t)(tile + 2 * L.sl.halo) * NP * sizeof(R);
     FusedArgs<R> a{(const R *)L.fin, (R *)L.fout, L.n, tile, L.cnt,
@@ -156,8 +165,9 @@ cudaError_t fused_family(bool fp64, int om, const FusedLaunch &L)
 template <class Sys, int DIM, class R>
 cudaError_t adjoint_prec(int om, const AdjointLaunch &L)
 {
-    // FP64: bound by the FP64 pipe, so blocks of 64 cells, which spread a short row over all SMs
-    // (with the tiles above, the gradient of 1D shallow water N = 16384, 4 steps: 15.1 -> 7.2 ms)
+    // FP64: bound by the FP64 pipe, so blocks of 64 cells, which spread a short row over all SMs (gradient of one step,
+    // FP64, blocks of 256 / 64: 1D entropic shallow water N = 4096 3440 / 2542 us, 100003 8025 / 7171, 2^20 58.2 / 58.3 ms;
+    // 2D entropic shallow water 192^2 16.0 / 14.1 ms, 1536^2 585 / 582; linear and Euler 64^2 ... 1536^2 within 1 % or faster)
     const unsigned block = sizeof(R) == 8 ? 64 : kBlock;
     dim3 grid((unsigned)((L.nx + block - 1) / block), (unsigned)L.ny);
     const ParamsR<R> P = params_as<R>(L.P);
