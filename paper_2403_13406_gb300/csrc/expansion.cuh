@@ -19,14 +19,18 @@
 //    and across it the kinetic energy adds (h_t - v_t h_1)^2 / (2 f_1 (1 + eta)).  Psi is stationary, so beta to
 //    order t^2 (beta_1, beta_2) gives B_k through t^5.
 //
-// The terms left out are bounded by the `size` of the cell, the ratio of successive terms: up to
-// Expansion::most the root of the truncated H is the root to the rounding of omega.  Rougher cells
+// The terms left out are bounded by the `size` of the cell, the ratio of successive terms: up to `most` (of
+// SmoothRoot and Expansion) the root of the truncated H is the root to the rounding of omega.  Rougher cells
 // take rough_root: Newton on B(t) - B(-1) from the truncated root, with B in the forms above (for
 // shallow water z = (eta + beta) / (1 - beta), (1 + z)(1 - beta) = 1 + eta, turns the stationarity of Psi into a
 // cubic in z), and what that does not certify, the general safeguarded search (entropic_omega).
-// Worst error of omega over 300 000 random cells per system (deviations of 1e-6 ... 0.5 of f), against a
-// bisection in long double: the expansion up to `most` 3e-7 in FP32 and 4e-16 in FP64, Newton on the closed
-// form 1e-6 (1.7e-5 next to the domain's edge) and 2e-15 (5e-14).
+// Worst error of omega over 60 000 random cells per system (1D and 2D shallow water and Burgers, deviations of 1e-7 ...
+// 0.5 of f, states up to the edge of the domain), against a bisection in 113 bits, by the cell's place in the domain
+// ((|v| + sqrt(g h)) / nu, or |c u| / V q / 2, below 0.9 / 0.99 / 0.999 / 0.99999):
+//   FP32  smooth  6e-8 / 2e-7 / 2e-6 / 1e-5    rough  6e-6 / 4e-6 / 6e-5 / 6e-4    general search  3e-3 / 2e-3 / 3e-2 / 1
+//   FP64  smooth  4e-17 / 9e-17 / 3e-16 / 2e-15   rough  1.2e-14 / 5e-15 / 7e-14 / 1e-12   general  2e-14 / 3e-14 / 3e-13 / 3e-2
+// Both round to nearest: next to the edge the diagnostics' bar of 64 roundings (7.6e-6 in FP32) is exceeded in 0.1 % of
+// such cells, on the general search alone in 1.3 %.
 //
 // The root-find bounds every entropic kernel (instruction issue in FP32, the FP64 pipe, 2 lanes a clock
 // and SM, in FP64).  Two evaluations of B by inner Newton solves, a quartic model through them and its
@@ -155,11 +159,10 @@ template <class Sys, class R> struct Expansion;
 template <int DIM, class R> struct Expansion<Scalar<DIM, true>, R> {
     static constexpr int Q = Lattice<DIM>::Q;
     static constexpr int N = sizeof(R) == 4 ? 6 : 8;
-    static constexpr int STEPS = sizeof(R) == 4 ? 0 : 1;
-    // largest size at which the terms left out (95 y^7 of c_2 in FP32, 286 y^8 in FP64) and the model root's
-    // own error (y^5 / 4; in FP64 after one Newton step y^7) are below the rounding of omega; beyond most_rough
+    // largest size at which the terms left out (286 y^8 of c_2) and the root's own error after one Newton step (y^7)
+    // are below the FP64 rounding of omega (the mixed mode's evaluation; SmoothRoot holds FP32's); beyond most_rough
     // (4 y -> 1: the edge of the domain) the closed form does not help
-    static constexpr R most = sizeof(R) == 4 ? R(0.04) : R(0.004);
+    static constexpr R most = R(0.004);
     static constexpr R most_rough = R(0.2);
     R c[N], size;
     R a[Q], y[Q];
@@ -219,10 +222,8 @@ template <int DIM, class R> struct Expansion<Scalar<DIM, true>, R> {
 template <int DIM, class R> struct Expansion<ShallowWater<DIM>, R> {
     static constexpr int Q = Lattice<DIM>::Q, M = DIM + 1;
     static constexpr int N = 4;
-    // sizes measured as above: at most, the error is 2e-7 (FP32) and 1e-16 (FP64); three times that size
-    // multiplies it by 3^5
-    static constexpr int STEPS = sizeof(R) == 4 ? 0 : 1;
-    static constexpr R most = sizeof(R) == 4 ? R(0.02) : R(3e-4);
+    // sizes measured as above: at most, the error is 1e-16 in FP64; three times that size multiplies it by 3^5
+    static constexpr R most = R(3e-4);
     static constexpr R most_rough = R(2);
     R c[N], size;
     R kap[Q], cv[Q], eta[Q], rr[Q], w[Q], zt[Q], z1[Q], z2[Q];
@@ -386,9 +387,7 @@ template <class R> __host__ __device__ __forceinline__ Two<R> rcp2(const Two<R> 
 // the sum of squares sq of the terms' ratios.  Very smooth cells (FP32, up to `few`: the terms of order
 // size^3 in omega are below its rounding) need c_2 and c_3 only: e = -c_3 / (c_2 + c_3).  c_2 scales with the square of
 // the fields (h V^2 size^2 for shallow water): in thin films, h of 1e-21 and below in FP32, it is subnormal while the
-// deviation is ordinary, rcp_fast takes it for zero and e is infinite or NaN, which omega_of refuses.  Worst error of omega on the
-// random cells above: FP32 scalar 4e-8 up to `few` and up to `most`, shallow water 5e-8 up to `few`, 1e-6 up to
-// `most` (next to the domain's edge; what Newton on the closed form gives there too), FP64 6e-17.
+// deviation is ordinary, rcp_fast takes it for zero and e is infinite or NaN, which omega_of refuses.
 template <class Sys, class R> struct SmoothRoot;
 
 template <int DIM, class R> struct SmoothRoot<Scalar<DIM, true>, R> {

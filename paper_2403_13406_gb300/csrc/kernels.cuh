@@ -193,7 +193,7 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
         bool found = false;
         // (FP64 coefficients of FP32 data are never subnormal)
         if (x.build(Pd, ud, dd) && x.size <= X::most) {
-            wd = x.size <= Eps<double>::value / 16.0 ? 2.0 : 2.0 + expansion_root<double, X::N>(x.c, X::STEPS);
+            wd = x.size <= Eps<double>::value / 16.0 ? 2.0 : 2.0 + expansion_root<double, X::N>(x.c, 1);
             found = wd < 1.0 + Pd.t_max;
         } else {
             found = rough_root<Sys, double>(Pd, ud, dd, wd);
