@@ -148,9 +148,10 @@ def aggregate(total_ms, units_per_rank, dist=None, device=None):
 # DRAM bytes (read + write) per launch of the dominant kernels, from the ncu captures summarised under
 # profiles/ (at a smaller size where noted, scaled by the cells a launch processes)
 TRAFFIC = {
-    "k_step2d_euler_8192_g2": (8.20e9, "profiles/k_step2d_euler_n2048_g2.txt: 513 MB at 2048^2, x 16"),
+    "k_step2d_euler_8192_g2": (8.30e9, "profiles/k_step2d_euler_n2048_g2.txt: 519 MB at 2048^2, x 16"),
     "k_stage_bulk_euler_8192": (7.70e9, "profiles/k_stage_bulk_euler_n2048_fp32_fixed.txt: 481 MB at 2048^2, x 16"),
-    "k_batch_step_sw2d_64": (47.0e9, "profiles/k_batch_step_sw2d_8inst_fp32_entropic.txt: 7.18 GB for 4.12 M cells, "
+    "k_step1d_sw1d_1m": (1.68e7, "profiles/k_step1d_sw1d_n1048576_fp32_entropic.txt: the state once, the writes stay in L2"),
+    "k_batch_step_sw2d_64": (47.3e9, "profiles/k_batch_step_sw2d_8inst_fp32_entropic.txt: 7.22 GB for 4.12 M cells, "
                                      "x 26.99 M / 4.12 M"),
 }
 
@@ -359,7 +360,7 @@ def timed_steps(torch, sim, stream, dev, n_steps, init=None):
 def sw1d_leg(torch, eslbm, inputs, stream, dev):
     """1D shallow water, N = 2^20, g = 9.81, V = 4, h0 = 1 + 0.1 sin 2 pi x, at rest, entropic omega,
     FP32 shifted by the state at rest, to t = 0.05 (8738 composite steps, one temporally blocked launch
-    each): throughput and the per-stage HBM model, with the ALU view of the entropic root-find."""
+    each): throughput and the per-stage HBM model (the kernel is bound by instruction issue, not by HBM)."""
     N = SW_N
     n_steps = inputs.steps_for(SW_T, 1.0 / N, SW_V)
     cfg = eslbm.make_config(1, "sw", N, V=SW_V, g=G, precision="fp32", omega_mode="entropic", u_ref=SW_UREF)
@@ -375,8 +376,7 @@ def sw1d_leg(torch, eslbm, inputs, stream, dev):
     sim.close()
     s = ms * 1e-3
     roof = hbm_roofline(18 * 2 * planes * 4, N * n_steps, s, "k_step1d<ShallowWater<1>, float, entropic>",
-                        n_steps,
-                        traffic=None)  # the capture predates the kernel's current D1Q2 deviations
+                        n_steps, traffic="k_step1d_sw1d_1m")
     return {"sw1d": {"workload": "sw1d_d1q2_entropic_n%d_t%g" % (N, SW_T), "N": N, "V": SW_V, "g": G,
                      "t_final": n_steps * 24.0 / N / SW_V, "composite_steps": n_steps, "ms": ms,
                      "site_updates_per_s": N * n_steps / s, "roofline": roof, "fallbacks": fb,
@@ -831,7 +831,7 @@ def profile_leg(torch, eslbm, inputs, stream, dev, case="euler", n=None, steps=2
     elif case.startswith("euler"):
         N = n or 2048
         cfg = eslbm.make_config(2, "euler", N, N, V=EULER_V, gamma=EULER_GAMMA, precision="fp32", omega_mode="fixed",
-                                blocking=group if case.endswith("blocked") else True)
+                                blocking=group if case.endswith("blocked") else False)
         u0 = inputs.euler_vortex_2d(N, N)
     else:
         N = n or BURGERS_N
