@@ -34,10 +34,10 @@
 //
 // The root-find bounds every entropic kernel (instruction issue in FP32, the FP64 pipe, 2 lanes a clock
 // and SM, in FP64).  Two evaluations of B by inner Newton solves, a quartic model through them and its
-// certificate took 652 thread instructions per 1D shallow-water cell-stage in all; with the expansion 305.
+// certificate took 652 thread instructions per 1D shallow-water cell-stage in all; with the expansion 299.
 // Before -> after: 1D shallow water N = 2^20, FP32, 409 -> 186 us per step; 2D Burgers 4096^2, FP32, 296 -> 141 us
 // per stage; 1D shallow water N = 100003, FP64, 3.26 -> 0.82 ms per step.  With the populations in packed pairs and
-// two coefficients for very smooth cells (SmoothRoot) 139 us per step and 110 us per stage (FP32).
+// two coefficients for very smooth cells (SmoothRoot) 215 instructions, 137 us per step and 110 us per stage (FP32).
 #pragma once
 
 #include "systems.cuh"

@@ -201,7 +201,7 @@ __device__ R mixed_omega(const ParamsR<R> &P, const R *u, const R *delta, R w, b
         if (found) {
             wd -= x.size * 0x1p-20;
             if (double(w) > wd) w = __double2float_rz(wd);
-            if (x.size <= 0.25) return w;
+            if (__double2hiint(x.size) < (1021 << 20)) return w;  // size < 0.25, off the FP64 pipe
         }
         typename Sys::template Ctx<double> cx;
         Sys::template prepare<double>(Pd, ud, dd, cx);
